@@ -74,7 +74,7 @@ def peaks():
 
 def kernel_source_hash():
     h = hashlib.sha256()
-    for f in ("gp_fft.cuh", "gp_sweep.cuh", "gp_tma.cuh", "gp_plane.cuh"):
+    for f in ("gp_fft.cuh", "gp_sweep.cuh", "gp_tma.cuh", "gp_warp.cuh", "gp_plane.cuh"):
         with open(os.path.join(ROOT, "paper_2003_03590_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

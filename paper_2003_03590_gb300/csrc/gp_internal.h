@@ -135,7 +135,7 @@ template <typename T> cudaError_t launch_vjp_nonlinear(const cpx<T>* psi_in, cpx
                                                        double shift, cudaStream_t s);
 
 // sweep variants (gp_step.cu): 0 TMA persistent, 1 TMA one CTA per SM, 2 plain, 3 TMA with two
-// stages, 4 TMA with two compute groups per CTA (lengths >= 512); for OP_PLANE 0 means the fused
+// stages, 4 TMA with another split into stages and compute groups (lengths >= 512); for OP_PLANE 0 means the fused
 // plane kernel, 3 the same with two stages and 2 the three separate sweeps it replaces
 enum { VARIANT_TMA = 0, VARIANT_TMA_ONE = 1, VARIANT_PLAIN = 2, VARIANT_TMA_2STAGE = 3, VARIANT_TMA_GROUPS = 4 };
 int sweep_variant(gp_plan* p, int n, int axis, int op);

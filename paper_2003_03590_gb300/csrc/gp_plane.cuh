@@ -35,13 +35,14 @@
 // launch can always proceed.  Every wait is bounded; a wait that gives up sets the status
 // word (the result is then invalid, the launch still ends).
 #pragma once
-#include "gp_tma.cuh"
+#include "gp_warp.cuh"
 
 namespace gp {
 
 struct TmaPlaneArgs {
   CUtensorMap map_y[GP_MAXB];   // per field: boxes of B x-columns by (up to 256) y
   CUtensorMap map_x[GP_MAXB];   // per field: boxes of (up to 256) x by B rows
+  float2* psi[GP_MAXB];         // the fields themselves (row copies of the warp-private kernels)
   int count;                    // fields
   const tw_t<float>* tw_fwd;
   const tw_t<float>* tw_inv;
@@ -60,12 +61,17 @@ struct TmaPlaneArgs {
 template <int L, int NS = 3, int NG = 1> struct TmaPlane {
   static constexpr int B = TmaStrided<L>::B;               // pencils (columns or rows) per tile
   static constexpr int TP = L / Plan<L>::E;                // threads per pencil
+  // pencils private to a warp (gp_warp.cuh): rows at a padded pitch, swizzled column tiles (which
+  // want stages on 1 KB boundaries); otherwise rows use a padded exchange layout
+  static constexpr bool WARP = warp_ok<L>();
   static constexpr int NC = B * TP;                        // compute threads of one group
   static constexpr int NT = NG * NC + 64;                  // + a loader warp and a storer warp
   static constexpr int Q = L / B;                          // tiles per phase and plane
   static constexpr int TILE = B * L;                       // elements
-  static constexpr int STAGE_C = B * contig_pitch<L>();    // rows use a padded exchange layout
-  static constexpr int STAGE = ((STAGE_C > TILE ? STAGE_C : TILE) + 15) / 16 * 16;   // 128-byte multiple
+  static constexpr int NW = NC / 32;                       // compute warps per group
+  static constexpr int STAGE_C = B * (WARP ? WarpContig<WARP ? L : 256>::pitch() : contig_pitch<L>());
+  static constexpr int ALIGN = WARP ? 1024 : 128;          // bytes
+  static constexpr int STAGE = ((STAGE_C > TILE ? STAGE_C : TILE) * 8 + ALIGN - 1) / ALIGN * (ALIGN / 8);   // elements
   static constexpr int BOX = L > 256 ? 256 : L;
   static constexpr int NBOX = L / BOX;
   static constexpr int S = NS;
@@ -76,7 +82,7 @@ template <int L, int NS = 3, int NG = 1> struct TmaPlane {
   static constexpr int TWF = tw_size<L, false>(), TWI = tw_size<L, true>();
   static constexpr size_t TWB = TWS ? (size_t)(TWF + TWI) * 16 : 0;
   static_assert(NS <= 8, "barrier arrays hold 8 stages");
-  static constexpr size_t SMEM = (size_t)S * STAGE * 8 + 192 + 64 + TWB + 128;   // barriers, ring and counts, twiddles, slack
+  static constexpr size_t SMEM = (size_t)S * STAGE * 8 + 192 + 64 + TWB + ALIGN;   // barriers, ring and counts, twiddles, slack
 };
 
 __device__ __forceinline__ int ld_relaxed_gpu(const int* p) {
@@ -91,10 +97,6 @@ __device__ __forceinline__ void red_release_gpu_add(int* p, int v) {
 __device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait1() { asm volatile("cp.async.bulk.wait_group 1;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait2() { asm volatile("cp.async.bulk.wait_group 2;" ::: "memory"); }
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
-
 
 // Item order.  Blocks of Q items (one phase of one plane) are ordered by "group" g: group g
 // holds phase 0 of plane g, phase 1 of plane g - D and phase 2 of plane g - 2D (those that
@@ -144,7 +146,7 @@ __global__ void __launch_bounds__(TmaPlane<L, NS, NG>::NT, TmaPlane<L, NS, NG>::
   constexpr int NCT = NG * NC;                                             // compute threads of the CTA
   extern __shared__ __align__(128) unsigned char smraw[];
   const uint32_t base = smem_u32(smraw);
-  V* buf = reinterpret_cast<V*>(smraw + (((base + 127u) & ~127u) - base));
+  V* buf = reinterpret_cast<V*>(smraw + (((base + G::ALIGN - 1u) & ~(G::ALIGN - 1u)) - base));
   uint64_t* full = reinterpret_cast<uint64_t*>(buf + (size_t)S * STAGE);   // data of stage s landed
   uint64_t* empty = full + 8;                                              // compute of stage s done
   uint64_t* freed = full + 16;                                             // stage s stored (read)
@@ -156,7 +158,7 @@ __global__ void __launch_bounds__(TmaPlane<L, NS, NG>::NT, TmaPlane<L, NS, NG>::
   if (tid == 0) {
     for (int s = 0; s < S; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], NC);
+      mbar_init(&empty[s], G::WARP ? G::NW : NC);
       mbar_init(&freed[s], 1);
       issued[s] = 0;
     }
@@ -181,6 +183,18 @@ __global__ void __launch_bounds__(TmaPlane<L, NS, NG>::NT, TmaPlane<L, NS, NG>::
     const int f = u / L, z = u - f * L;
     V* st = buf + (size_t)s * STAGE;
     const uint64_t pol = (load ? ph == 0 : ph == 2) ? pol_first : pol_last;
+    if constexpr (G::WARP) {
+      if (ph == 1) {   // row by row, at the pitch of the exchange
+        float2* g = a.psi[f] + ((size_t)z * L + (size_t)j * B) * L;
+        uint32_t row = smem_u32(st);
+#pragma unroll
+        for (int q = 0; q < B; ++q, row += WarpContig<L>::pitch() * 8) {
+          if (load) bulk_load_hint(row, g + (size_t)q * L, L * 8, &full[s], pol);
+          else bulk_store_hint(g + (size_t)q * L, row, L * 8, pol);
+        }
+        return;
+      }
+    }
 #pragma unroll
     for (int k = 0; k < G::NBOX; ++k) {
       V* sk = st + (size_t)k * BOX * B;
@@ -327,6 +341,35 @@ __global__ void __launch_bounds__(TmaPlane<L, NS, NG>::NT, TmaPlane<L, NS, NG>::
   sa.ek2 = a.ek2;
   sa.scale_inv = 0;
   const int grp = tid / NC, lt = tid % NC;
+  if constexpr (G::WARP) {
+    const int lane = lt & 31;
+    WarpContig<L> AC(lt >> 5, lane);
+    WarpStrided<L, B> AS(lt >> 5, lane);
+    for (int k = grp;; k += NG) {
+      const int s = k % S;
+      const bool ok = NG > 1 ? stage_wait(&full[s], issued + s, k, S) : mbar_wait_bounded(&full[s], (unsigned)(k / S) & 1u);
+      if (!__all_sync(0xffffffffu, ok)) {
+        if (lane == 0) atomicExch(a.status, 1);
+        break;
+      }
+      const int it = ring[s];
+      if (it < 0) break;
+      const int ph = it & 3, j = (it >> 2) & 511, z = (it >> 11) % L;
+      const uint32_t st = smem_u32(buf + (size_t)s * STAGE);
+      if (ph == 1) {
+        AC.at(st);
+        warp_op<OP_FWD_K_INV, L, WarpContig<L>, G::TWS>(sa, AC, j * B + AC.p, z);
+      } else {
+        AS.at(st);
+        if (ph == 0) warp_op<OP_FWD, L, WarpStrided<L, B>, G::TWS>(sa, AS, 0, 0);
+        else warp_op<OP_INV, L, WarpStrided<L, B>, G::TWS>(sa, AS, 0, 0);
+      }
+      fence_async_smem();      // this thread's writes of the stage, before the copy that reads them
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&empty[s]);
+    }
+    return;
+  }
   for (int k = grp;; k += NG) {
     const int s = k % S;
     // several groups: the stage may still serve an earlier item of another group; wait until the
@@ -374,8 +417,8 @@ __global__ void __launch_bounds__(TmaPlane<L, NS, NG>::NT, TmaPlane<L, NS, NG>::
 
 // compute groups and stages of the grouped plane kernel: 512: three groups, five stages;
 // 1024: two groups, three stages (a 1024-point stage is 70 KB)
-template <int L> __host__ __device__ constexpr int plane_groups() { return L >= 1024 ? 2 : 3; }
-template <int L> __host__ __device__ constexpr int plane_group_stages() { return L >= 1024 ? 3 : 5; }
+template <int L> __host__ __device__ constexpr int plane_groups() { return L >= 1024 ? 2 : 4; }
+template <int L> __host__ __device__ constexpr int plane_group_stages() { return L >= 1024 ? 3 : 6; }
 
 template <int L> struct TmaPlaneLaunch {
   template <int NS, int NG> static int occupancy() {

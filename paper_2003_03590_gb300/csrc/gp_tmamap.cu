@@ -37,29 +37,30 @@ template <int L> static void box_of(int axis, cuuint32_t box[3]) {
   } else if (axis == 1) {
     box[0] = TmaStrided<L>::B; box[1] = TmaStrided<L>::BOX; box[2] = 1;
   } else {
-    box[0] = TmaStrided<L, 3, z_wide<L>()>::B; box[1] = 1; box[2] = TmaStrided<L>::BOX;
+    box[0] = warp_z_pencils<L>(); box[1] = 1; box[2] = TmaStrided<L>::BOX;
   }
 }
 
-template <int L> static bool swizzled(int axis) { return axis != 0 && TmaStrided<L>::SWZ; }
+// y/z tiles of the warp-private kernels are swizzled by their row length (64 or 128 bytes)
+template <int L> static int swizzle_of(bool warp, const cuuint32_t box[3]) { return warp ? (int)box[0] * 8 : 0; }
 
-static bool encode_box(CUtensorMap* m, void* base, int n, const cuuint32_t box[3], bool swz) {
+static bool encode_box(CUtensorMap* m, void* base, int n, const cuuint32_t box[3], int swz) {
   auto enc = encode_fn();
   if (!enc) return false;
   cuuint64_t dims[3] = {(cuuint64_t)n, (cuuint64_t)n, (cuuint64_t)n};
   cuuint64_t strides[2] = {(cuuint64_t)n * 8, (cuuint64_t)n * n * 8};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = enc(m, CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                   swz ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                   swz == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : swz == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
 
 static bool make_map(CUtensorMap* m, void* base, int n, int axis) {
   cuuint32_t box[3];
-  bool swz = false;
+  int swz = 0;
   switch (n) {
-#define GP_CASE(L) case L: box_of<L>(axis, box); swz = swizzled<L>(axis); break;
+#define GP_CASE(L) case L: box_of<L>(axis, box); swz = swizzle_of<L>(axis != 0 && warp_axis<L>(axis), box); break;
     GP_TMA_SIZES(GP_CASE)
 #undef GP_CASE
     default: return false;
@@ -77,6 +78,7 @@ cudaError_t tma_sweep(int n, const SweepArgs<float>& a, void* const* psi, int* s
   t.count = a.count;
   for (int f = 0; f < a.count; ++f)
     if (!make_map(&t.map[f], psi[f], n, a.axis)) return cudaErrorInvalidValue;
+  for (int f = 0; f < a.count; ++f) t.psi[f] = (float2*)psi[f];
   t.tw_fwd = a.tw_fwd;
   t.tw_inv = a.tw_inv;
   t.ekx = a.ekx;
@@ -104,11 +106,13 @@ cudaError_t tma_plane(int n, const SweepArgs<float>& a, void* const* psi, int* s
   std::memset(&t, 0, sizeof(t));
   t.count = a.count;
   cuuint32_t by[3], bx[3];
+  int swz = 0;
   switch (n) {
 #define GP_CASE(L)                                                                          \
   case L:                                                                                   \
     by[0] = TmaPlane<L>::B; by[1] = TmaPlane<L>::BOX; by[2] = 1;                            \
     bx[0] = TmaPlane<L>::BOX; bx[1] = TmaPlane<L>::B; bx[2] = 1;                            \
+    swz = swizzle_of<L>(warp_ok<L>(), by);                                                           \
     break;
     GP_TMA_SIZES(GP_CASE)
 #undef GP_CASE
@@ -116,8 +120,9 @@ cudaError_t tma_plane(int n, const SweepArgs<float>& a, void* const* psi, int* s
       return cudaErrorInvalidValue;
   }
   for (int f = 0; f < a.count; ++f)
-    if (!encode_box(&t.map_y[f], psi[f], n, by, false) || !encode_box(&t.map_x[f], psi[f], n, bx, false))
+    if (!encode_box(&t.map_y[f], psi[f], n, by, swz) || !encode_box(&t.map_x[f], psi[f], n, bx, 0))
       return cudaErrorInvalidValue;
+  for (int f = 0; f < a.count; ++f) t.psi[f] = (float2*)psi[f];
   t.tw_fwd = a.tw_fwd;
   t.tw_inv = a.tw_inv;
   t.ekx = a.ekx;

@@ -46,8 +46,9 @@ typedef enum {
 typedef enum { GP_FP32 = 0, GP_FP64 = 1 } gp_precision;
 /* GP_FP32: complex64 storage, fused sweeps (the nonlinear phase is applied
  *          inside the FFT sweeps, the kinetic propagator inside the middle sweep).
- * GP_FP64: complex128 storage, plain unfused path (one kernel per sub-flow and
- *          per FFT axis), the accuracy reference on the GPU. */
+ * GP_FP64: complex128 storage, the same fused sweeps in 64-bit fixed point per
+ *          pencil (more accurate than float64 transforms, and this GPU has few
+ *          float64 units), the accuracy reference on the GPU. */
 
 typedef enum { GP_SPLIT_NKN = 0, GP_SPLIT_KNK = 1 } gp_split;
 /* NKN: psi' = N(dt/2) K(dt) N(dt/2) psi, consecutive half steps merged.

@@ -196,10 +196,10 @@ template <typename T> static gp_status adjoint_impl(gp_plan* p, int field, const
   cpx<T>* tmp = S + (size_t)nsteps * npts;
   const double dt = F.prm.dt, h = 0.5 * dt, shift = F.prm.nonlin_minus_one ? 1.0 : 0.0;
   const bool f64 = sizeof(T) == 8;
-  const cpx<T>* kd = (const cpx<T>*)ktable(p, field, dt, f64);
-  const cpx<T>* kmd = (const cpx<T>*)ktable(p, field, -dt, f64);
-  const cpx<T>* kh = (const cpx<T>*)ktable(p, field, h, f64);
-  const cpx<T>* kmh = (const cpx<T>*)ktable(p, field, -h, f64);
+  const void* kd = ktable(p, field, dt, f64);
+  const void* kmd = ktable(p, field, -dt, f64);
+  const void* kh = ktable(p, field, h, f64);
+  const void* kmh = ktable(p, field, -h, f64);
   if (!kd || !kmd || !kh || !kmh) return fail(p, GP_ERR_OOM, "kinetic table allocation");
   // recompute the states at the start of every step of the segment
   GP_CUDA(p, cudaMemcpyAsync(S, psi_n, fb, cudaMemcpyDeviceToDevice, s));

@@ -4,7 +4,6 @@
 
 namespace gp {
 cudaError_t sweep_f32_256(const SweepArgs<float>& a, cudaStream_t s) { return SweepLaunch<float, 256>::launch(a, s); }
-cudaError_t sweep_f64_256(const SweepArgs<double>& a, cudaStream_t s) { return SweepLaunch<double, 256>::launch(a, s); }
 cudaError_t tma_sweep_256(const TmaSweepArgs& a, int ctas, int stages, int groups, cudaStream_t s) {
   return WarpLaunch<256>::launch(a, ctas, stages, groups, s);
 }

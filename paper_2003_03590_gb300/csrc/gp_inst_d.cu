@@ -4,7 +4,6 @@
 
 namespace gp {
 cudaError_t sweep_f32_512(const SweepArgs<float>& a, cudaStream_t s) { return SweepLaunch<float, 512>::launch(a, s); }
-cudaError_t sweep_f64_512(const SweepArgs<double>& a, cudaStream_t s) { return SweepLaunch<double, 512>::launch(a, s); }
 cudaError_t tma_sweep_512(const TmaSweepArgs& a, int ctas, int stages, int groups, cudaStream_t s) {
   return WarpLaunch<512>::launch(a, ctas, stages, groups, s);
 }

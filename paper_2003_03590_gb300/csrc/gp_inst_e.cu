@@ -4,7 +4,6 @@
 
 namespace gp {
 cudaError_t sweep_f32_1024(const SweepArgs<float>& a, cudaStream_t s) { return SweepLaunch<float, 1024>::launch(a, s); }
-cudaError_t sweep_f64_1024(const SweepArgs<double>& a, cudaStream_t s) { return SweepLaunch<double, 1024>::launch(a, s); }
 cudaError_t tma_sweep_1024(const TmaSweepArgs& a, int ctas, int stages, int groups, cudaStream_t s) {
   return WarpLaunch<1024>::launch(a, ctas, stages, groups, s);
 }

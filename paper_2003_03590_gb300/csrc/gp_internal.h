@@ -6,14 +6,14 @@
 #include <vector>
 
 #include "gp.h"
-#include "gp_sweep.cuh"
+#include "gp_fixsweep.cuh"
 
 namespace gp {
 
 #define GP_SIZES(X) X(8) X(12) X(16) X(24) X(32) X(48) X(64) X(96) X(128) X(192) X(256) X(512) X(1024)
 #define GP_DECL_SWEEP(L)                                                   \
   cudaError_t sweep_f32_##L(const SweepArgs<float>&, cudaStream_t);        \
-  cudaError_t sweep_f64_##L(const SweepArgs<double>&, cudaStream_t);
+  cudaError_t sweep_f64_##L(const FixArgs&, cudaStream_t);
 GP_SIZES(GP_DECL_SWEEP)
 #undef GP_DECL_SWEEP
 
@@ -51,12 +51,13 @@ void split_hilo(double v, float* hi, float* lo);   // see gp_plan.cu
 int plan_np(int n);           // number of radix passes for length n
 int plan_radix_fwd(int n, int i);
 cudaError_t sweep(int n, const SweepArgs<float>& a, cudaStream_t s);
-cudaError_t sweep(int n, const SweepArgs<double>& a, cudaStream_t s);
+cudaError_t sweep(int n, const FixArgs& a, cudaStream_t s);
 
 // Device tables of one grid length in one precision.
 struct Tables {
   void* tw_fwd = nullptr;  // Stockham twiddles, forward direction
   void* tw_inv = nullptr;  // inverse direction
+  void* dir = nullptr;     // float64: the 256 directions of the nonlinear phase (gp_fix.cuh)
 };
 
 // Kinetic propagator table exp(-i alpha k^2 s) for a given s, per storage type.
@@ -125,12 +126,13 @@ gp_status ensure_ws(gp_plan* p, int field, size_t bytes);
 // 3D transforms of a whole field through the pencil sweeps (unfused).
 template <typename T> cudaError_t fft3(FieldPlan& F, cpx<T>* x, bool inverse, cudaStream_t s);
 // K with fused sweeps: fwd z, fwd y, [fwd x, K (table ek), 1/N^3, inv x], inv y, inv z.
-template <typename T> cudaError_t kinetic3(FieldPlan& F, cpx<T>* x, const cpx<T>* ek, cudaStream_t s);
-template <typename T> const Tables& tables(FieldPlan& F);
+// ek: the table that ktable returns
+template <typename T> cudaError_t kinetic3(FieldPlan& F, cpx<T>* x, const void* ek, cudaStream_t s);
+// the tables of a float64 field's sweeps (ek: from ktable, or null)
+FixArgs fix_args(FieldPlan& F, const void* ek);
 
 // pointwise kernels (gp_pointwise.cu)
 template <typename T> cudaError_t launch_nonlinear(cpx<T>* psi, long long npts, double coef, double shift, cudaStream_t s);
-template <typename T> cudaError_t launch_kinetic_mul(cpx<T>* psi, int n, const cpx<T>* ek, cudaStream_t s);
 template <typename T> cudaError_t launch_vjp_nonlinear(const cpx<T>* psi_in, cpx<T>* lam, long long npts, double coef,
                                                        double shift, cudaStream_t s);
 

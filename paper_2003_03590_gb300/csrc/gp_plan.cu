@@ -47,7 +47,7 @@ cudaError_t sweep(int n, const SweepArgs<float>& a, cudaStream_t s) {
     default: return cudaErrorInvalidValue;
   }
 }
-cudaError_t sweep(int n, const SweepArgs<double>& a, cudaStream_t s) {
+cudaError_t sweep(int n, const FixArgs& a, cudaStream_t s) {
   switch (n) {
 #define GP_CASE(L) case L: return sweep_f64_##L(a, s);
     GP_SIZES(GP_CASE)
@@ -127,8 +127,49 @@ template <> float4 pack<float4>(double c, double s) {
   split_hilo(s, &sh, &sl);
   return make_float4(ch, sh, cl, sl);
 }
-template <> double2 pack<double2>(double c, double s) { return make_double2(c, s); }
-template <> float2 pack<float2>(double c, double s) { return make_float2((float)c, (float)s); }
+// float64: fixed point, (c + 1) / 2 and (s + 1) / 2 in units of 2^-64, even
+template <> ufix2 pack<ufix2>(double c, double s) {
+  auto u = [](double v) {
+    const double w = std::ldexp(v, 62);                        // exact; |v| <= 1
+    const long long q = (long long)std::nearbyint(w);
+    const unsigned long long r = ((unsigned long long)q << 1) + (1ull << 63);   // (v + 1) 2^63
+    return v >= 1.0 ? ~1ull : r;
+  };
+  return ufix2{u(c), u(s)};
+}
+
+// cos and sin of 2 pi num / den (0 <= num < den) to about 2^-60: the angle is reduced to the first
+// octant in integers and the Taylor series summed in units of 2^-60
+static ufix2 direction(long long num, long long den, bool neg_sin) {
+  typedef unsigned __int128 u128;
+  int oct = (int)(8 * num / den);                              // octant of the angle
+  long long a = 8 * num - oct * den, b = den;                  // remaining fraction a / b of an octant
+  if (oct & 1) a = b - a;                                      // measured from the nearer axis
+  const u128 pi4 = 0xC90FDAA22168C235ull;                      // pi / 4 2^64
+  const unsigned long long th = (unsigned long long)((pi4 * (u128)a / (u128)b) >> 4);   // 2^-60
+  auto mul = [](unsigned long long x, unsigned long long y) { return (unsigned long long)(((u128)x * y + ((u128)1 << 59)) >> 60); };
+  const unsigned long long one = 1ull << 60, z = mul(th, th);
+  long long c = (long long)one, s = (long long)th;
+  unsigned long long tc = one, ts = th;
+  for (int k = 1; k <= 11; ++k) {
+    tc = mul(tc, z) / (unsigned long long)((2 * k - 1) * (2 * k));
+    ts = mul(ts, z) / (unsigned long long)((2 * k) * (2 * k + 1));
+    c += (k & 1) ? -(long long)tc : (long long)tc;
+    s += (k & 1) ? -(long long)ts : (long long)ts;
+  }
+  // octants 1, 2, 5, 6: measured from the imaginary axis
+  const int o = oct;
+  long long re, im;
+  if (o == 1 || o == 2 || o == 5 || o == 6) { re = s; im = c; } else { re = c; im = s; }
+  if (o >= 2 && o <= 5) re = -re;
+  if (o >= 4) im = -im;
+  if (neg_sin) im = -im;
+  auto u = [&](long long v) {
+    const unsigned long long r = ((unsigned long long)v << 3) + (1ull << 63);
+    return v >= (long long)one ? ~1ull : r;
+  };
+  return ufix2{u(re), u(im)};
+}
 
 template <typename V> static cudaError_t upload(const std::vector<double>& re, const std::vector<double>& im, void** dev) {
   std::vector<V> h(re.size() > 0 ? re.size() : 1);
@@ -138,6 +179,12 @@ template <typename V> static cudaError_t upload(const std::vector<double>& re, c
   return cudaMemcpy(*dev, h.data(), h.size() * sizeof(V), cudaMemcpyHostToDevice);
 }
 
+static cudaError_t upload_raw(const std::vector<ufix2>& h, void** dev) {
+  cudaError_t e = cudaMalloc(dev, (h.empty() ? 1 : h.size()) * sizeof(ufix2));
+  if (e != cudaSuccess || h.empty()) return e;
+  return cudaMemcpy(*dev, h.data(), h.size() * sizeof(ufix2), cudaMemcpyHostToDevice);
+}
+
 static cudaError_t build_tables(FieldPlan& F) {
   std::vector<double> re, im;
   cudaError_t e;
@@ -145,10 +192,20 @@ static cudaError_t build_tables(FieldPlan& F) {
     twiddles(F.n, inv != 0, re, im);
     e = upload<float4>(re, im, inv ? &F.t32.tw_inv : &F.t32.tw_fwd);
     if (e != cudaSuccess) return e;
-    e = upload<double2>(re, im, inv ? &F.t64.tw_inv : &F.t64.tw_fwd);
+    std::vector<ufix2> tw;
+    const int np = plan_np(F.n);
+    for (int i = 0, ns = 1; i < np; ++i) {
+      const int R = plan_radix_fwd(F.n, inv ? np - 1 - i : i);
+      for (int jm = 0; jm < ns; ++jm)
+        for (int r = 1; r < R; ++r) tw.push_back(direction(((long long)r * jm) % ((long long)ns * R), (long long)ns * R, inv == 0));
+      ns *= R;
+    }
+    e = upload_raw(tw, inv ? &F.t64.tw_inv : &F.t64.tw_fwd);
     if (e != cudaSuccess) return e;
   }
-  return cudaSuccess;
+  std::vector<ufix2> dir(256);
+  for (int k = 0; k < 256; ++k) dir[k] = direction(k, 256, false);
+  return upload_raw(dir, &F.t64.dir);
 }
 
 // exp(-i alpha k^2 s) for grid index i (k = i for i < N/2, else i - N; Nyquist k^2 = (N/2)^2).
@@ -164,9 +221,9 @@ static void ktable_values(int n, double alpha, double s, std::vector<double>& re
   }
 }
 
-// float64 fields: N entries exp(-i alpha k^2 s).  float32 fields: N hi/lo entries of the same,
-// followed by N^2 hi/lo entries of exp(-i alpha (k1^2 + k2^2) s) / N^3 (index i2 N + i1),
-// each formed in float64 and split into hi + lo.
+// N entries exp(-i alpha k^2 s), followed by N^2 entries of exp(-i alpha (k1^2 + k2^2) s) nu (index
+// i2 N + i1), formed in float64.  float32 fields: hi/lo pairs, nu = 1/N^3; float64 fields: fixed point,
+// nu = 1 or, for lengths 3 2^k, 16/27 (the powers of two of 1/N^3 go into the sweep's scale).
 const void* ktable(gp_plan* p, int field, double s, bool fp64) {
   FieldPlan& F = p->f[field];
   std::vector<KTable>& cache = fp64 ? F.k64 : F.k32;
@@ -177,11 +234,9 @@ const void* ktable(gp_plan* p, int field, double s, bool fp64) {
   KTable kt;
   kt.s = s;
   cudaError_t e;
-  if (fp64) {
-    e = upload<double2>(re, im, &kt.dev);
-  } else {
+  {
     const int n = F.n;
-    const double norm = 1.0 / (double)F.npts;
+    const double norm = !fp64 ? 1.0 / (double)F.npts : (n % 3 == 0 ? 16.0 / 27.0 : 1.0);
     std::vector<double> r2((size_t)n + (size_t)n * n), i2((size_t)n + (size_t)n * n);
     for (int i = 0; i < n; ++i) {
       r2[i] = re[i];
@@ -193,7 +248,7 @@ const void* ktable(gp_plan* p, int field, double s, bool fp64) {
         r2[q] = (re[a] * re[b] - im[a] * im[b]) * norm;
         i2[q] = (re[a] * im[b] + im[a] * re[b]) * norm;
       }
-    e = upload<float4>(r2, i2, &kt.dev);
+    e = fp64 ? upload<ufix2>(r2, i2, &kt.dev) : upload<float4>(r2, i2, &kt.dev);
   }
   if (e != cudaSuccess) return nullptr;
   cache.push_back(kt);
@@ -212,16 +267,32 @@ gp_status ensure_ws(gp_plan* p, int field, size_t bytes) {
   return GP_OK;
 }
 
-template <> const Tables& tables<float>(FieldPlan& F) { return F.t32; }
-template <> const Tables& tables<double>(FieldPlan& F) { return F.t64; }
+FixArgs fix_args(FieldPlan& F, const void* ek) {
+  FixArgs a{};
+  a.count = 1;
+  a.tw_fwd = (const ufix2*)F.t64.tw_fwd;
+  a.tw_inv = (const ufix2*)F.t64.tw_inv;
+  a.dir = (const ufix2*)F.t64.dir;
+  a.ek = (const ufix2*)ek;
+  return a;
+}
+static SweepArgs<float> f32_args(FieldPlan& F, const void* ek) {
+  SweepArgs<float> a{};
+  a.count = 1;
+  a.tw_fwd = (const tw_t<float>*)F.t32.tw_fwd;
+  a.tw_inv = (const tw_t<float>*)F.t32.tw_inv;
+  a.ekx = (const float4*)ek;
+  if (ek) a.ek2 = (const float4*)ek + F.n;
+  return a;
+}
+template <typename T> static auto sweep_args(FieldPlan& F, const void* ek) {
+  if constexpr (sizeof(T) == 4) return f32_args(F, ek);
+  else return fix_args(F, ek);
+}
 
 template <typename T> cudaError_t fft3(FieldPlan& F, cpx<T>* x, bool inverse, cudaStream_t s) {
-  const Tables& tb = tables<T>(F);
-  SweepArgs<T> a{};
+  auto a = sweep_args<T>(F, nullptr);
   a.psi[0] = x;
-  a.count = 1;
-  a.tw_fwd = (const tw_t<T>*)tb.tw_fwd;
-  a.tw_inv = (const tw_t<T>*)tb.tw_inv;
   a.op = inverse ? OP_INV : OP_FWD;
   a.scale_inv = 1;
   const int order_f[3] = {0, 1, 2}, order_i[3] = {2, 1, 0};
@@ -235,20 +306,9 @@ template <typename T> cudaError_t fft3(FieldPlan& F, cpx<T>* x, bool inverse, cu
 template cudaError_t fft3<float>(FieldPlan&, cpx<float>*, bool, cudaStream_t);
 template cudaError_t fft3<double>(FieldPlan&, cpx<double>*, bool, cudaStream_t);
 
-template <typename T> cudaError_t kinetic3(FieldPlan& F, cpx<T>* x, const cpx<T>* ek, cudaStream_t s) {
-  const Tables& tb = tables<T>(F);
-  SweepArgs<T> a{};
+template <typename T> cudaError_t kinetic3(FieldPlan& F, cpx<T>* x, const void* ek, cudaStream_t s) {
+  auto a = sweep_args<T>(F, ek);
   a.psi[0] = x;
-  a.count = 1;
-  a.tw_fwd = (const tw_t<T>*)tb.tw_fwd;
-  a.tw_inv = (const tw_t<T>*)tb.tw_inv;
-  if constexpr (sizeof(T) == 4) {
-    a.ekx = (const float4*)ek;
-    a.ek2 = (const float4*)ek + F.n;
-  } else {
-    a.ek = ek;
-    a.k_norm = kconst(1.0 / (double)F.npts);
-  }
   a.scale_inv = 0;
   const int axes[5] = {2, 1, 0, 1, 2};
   const int ops[5] = {OP_FWD, OP_FWD, OP_FWD_K_INV, OP_INV, OP_INV};
@@ -260,11 +320,11 @@ template <typename T> cudaError_t kinetic3(FieldPlan& F, cpx<T>* x, const cpx<T>
   }
   return cudaSuccess;
 }
-template cudaError_t kinetic3<float>(FieldPlan&, cpx<float>*, const cpx<float>*, cudaStream_t);
-template cudaError_t kinetic3<double>(FieldPlan&, cpx<double>*, const cpx<double>*, cudaStream_t);
+template cudaError_t kinetic3<float>(FieldPlan&, cpx<float>*, const void*, cudaStream_t);
+template cudaError_t kinetic3<double>(FieldPlan&, cpx<double>*, const void*, cudaStream_t);
 
 static void free_field(FieldPlan& F) {
-  void* ptrs[] = {F.t32.tw_fwd, F.t32.tw_inv, F.t64.tw_fwd, F.t64.tw_inv, F.host_buf, F.ws};
+  void* ptrs[] = {F.t32.tw_fwd, F.t32.tw_inv, F.t64.tw_fwd, F.t64.tw_inv, F.t64.dir, F.host_buf, F.ws};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   for (auto& k : F.k32)

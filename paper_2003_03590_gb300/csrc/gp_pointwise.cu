@@ -14,16 +14,6 @@ template <typename T> __global__ void k_nonlinear(cpx<T>* psi, long long npts, T
     psi[i] = nonlinear(psi[i], coef, shift);
 }
 
-// K in Fourier space: psi_k *= E[kx] E[ky] E[kz]
-template <typename T> __global__ void k_kinetic_mul(cpx<T>* psi, int n, const cpx<T>* __restrict__ ek) {
-  const long long npts = (long long)n * n * n;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < npts; i += (long long)gridDim.x * blockDim.x) {
-    int ix = (int)(i % n), iy = (int)((i / n) % n), iz = (int)(i / ((long long)n * n));
-    cpx<T> f = cmul(cmul(__ldg(ek + ix), __ldg(ek + iy)), __ldg(ek + iz));
-    psi[i] = cmul(psi[i], f);
-  }
-}
-
 // VJP of N(s) at input psi_in: lam <- exp(+i phi) lam + 2 coef Im(conj(lam) psi_out) psi_in,
 // phi = coef (|psi_in|^2 - shift), psi_out = exp(-i phi) psi_in, coef = beta s.
 template <typename T>
@@ -63,10 +53,6 @@ template <typename T> cudaError_t launch_nonlinear(cpx<T>* psi, long long npts, 
   k_nonlinear<T><<<grid_for(npts, 256), 256, 0, s>>>(psi, npts, (T)coef, (T)shift);
   return cudaGetLastError();
 }
-template <typename T> cudaError_t launch_kinetic_mul(cpx<T>* psi, int n, const cpx<T>* ek, cudaStream_t s) {
-  k_kinetic_mul<T><<<grid_for((long long)n * n * n, 256), 256, 0, s>>>(psi, n, ek);
-  return cudaGetLastError();
-}
 template <typename T>
 cudaError_t launch_vjp_nonlinear(const cpx<T>* psi_in, cpx<T>* lam, long long npts, double coef, double shift, cudaStream_t s) {
   k_vjp_nonlinear<T><<<grid_for(npts, 256), 256, 0, s>>>(psi_in, lam, npts, (T)coef, (T)shift);
@@ -74,8 +60,6 @@ cudaError_t launch_vjp_nonlinear(const cpx<T>* psi_in, cpx<T>* lam, long long np
 }
 template cudaError_t launch_nonlinear<float>(cpx<float>*, long long, double, double, cudaStream_t);
 template cudaError_t launch_nonlinear<double>(cpx<double>*, long long, double, double, cudaStream_t);
-template cudaError_t launch_kinetic_mul<float>(cpx<float>*, int, const cpx<float>*, cudaStream_t);
-template cudaError_t launch_kinetic_mul<double>(cpx<double>*, int, const cpx<double>*, cudaStream_t);
 template cudaError_t launch_vjp_nonlinear<float>(const cpx<float>*, cpx<float>*, long long, double, double, cudaStream_t);
 template cudaError_t launch_vjp_nonlinear<double>(const cpx<double>*, cpx<double>*, long long, double, double, cudaStream_t);
 

@@ -13,7 +13,8 @@
 // (blockIdx.y selects the field), and the repeating four-sweep cycle is
 // captured once in a CUDA graph and replayed.
 //
-// float64 fields (plain): one kernel per sub-flow and per FFT axis, step by step.
+// float64 fields run the same four-sweep cycle with the sweeps of gp_fixsweep.cuh.  (One kernel per
+// sub-flow and axis, with unmerged half steps, took 9 or 15 launches and two N per step.)
 #include <cmath>
 #include <cstdio>
 #include <string>
@@ -162,6 +163,20 @@ std::vector<Group> make_groups(gp_plan* p) {
 
 gp_status launch_item(gp_plan* p, const Group& G, const Item& it, void* const* psi, cudaStream_t s) {
   FieldPlan& F = p->f[G.fields[0]];
+  if (G.fp64) {
+    const void* kt = nullptr;
+    if (it.op == OP_FWD_K_INV && !(kt = ktable(p, G.fields[0], it.s_k, true)))
+      return fail(p, GP_ERR_OOM, "kinetic table allocation");
+    FixArgs a = fix_args(F, kt);
+    a.count = (int)G.fields.size();
+    for (int k = 0; k < a.count; ++k) a.psi[k] = (double2*)psi[G.fields[k]];
+    a.op = it.op;
+    a.axis = it.axis;
+    a.nl = nl_fix(F.beta * it.s_nl, F.prm.nonlin_minus_one ? 1.0 : 0.0);
+    GP_CUDA(p, sweep(G.n, a, s));
+    p->launches += 1;
+    return GP_OK;
+  }
   SweepArgs<float> a{};
   a.count = (int)G.fields.size();
   for (int k = 0; k < a.count; ++k) a.psi[k] = (cpx<float>*)psi[G.fields[k]];
@@ -228,36 +243,6 @@ gp_status run_items(gp_plan* p, const std::vector<Group>& groups, const std::vec
   for (const Item& it : items) {
     gp_status st = launch_item(p, groups[it.group], it, psi, s);
     if (st != GP_OK) return st;
-  }
-  return GP_OK;
-}
-
-// plain float64 step of one field: N and K as separate kernels, 3D FFTs as three sweeps each
-gp_status plain_steps(gp_plan* p, int field, cpx<double>* psi, int nsteps) {
-  FieldPlan& F = p->f[field];
-  const double dt = F.prm.dt, h = 0.5 * dt;
-  const double shift = F.prm.nonlin_minus_one ? 1.0 : 0.0;
-  const cpx<double>* kd = (const cpx<double>*)ktable(p, field, dt, true);
-  const cpx<double>* kh = (const cpx<double>*)ktable(p, field, h, true);
-  if (!kd || !kh) return fail(p, GP_ERR_OOM, "kinetic table allocation");
-  cudaStream_t s = p->stream;
-  p->launches += (long long)nsteps * (F.prm.split == GP_SPLIT_NKN ? 9 : 15);
-  for (int m = 0; m < nsteps; ++m) {
-    if (F.prm.split == GP_SPLIT_NKN) {
-      GP_CUDA(p, launch_nonlinear<double>(psi, F.npts, F.beta * h, shift, s));
-      GP_CUDA(p, fft3<double>(F, psi, false, s));
-      GP_CUDA(p, launch_kinetic_mul<double>(psi, F.n, kd, s));
-      GP_CUDA(p, fft3<double>(F, psi, true, s));
-      GP_CUDA(p, launch_nonlinear<double>(psi, F.npts, F.beta * h, shift, s));
-    } else {
-      GP_CUDA(p, fft3<double>(F, psi, false, s));
-      GP_CUDA(p, launch_kinetic_mul<double>(psi, F.n, kh, s));
-      GP_CUDA(p, fft3<double>(F, psi, true, s));
-      GP_CUDA(p, launch_nonlinear<double>(psi, F.npts, F.beta * dt, shift, s));
-      GP_CUDA(p, fft3<double>(F, psi, false, s));
-      GP_CUDA(p, launch_kinetic_mul<double>(psi, F.n, kh, s));
-      GP_CUDA(p, fft3<double>(F, psi, true, s));
-    }
   }
   return GP_OK;
 }
@@ -384,34 +369,23 @@ gp_status step_all(gp_plan* p, void* const* psi, int nsteps) {
   if (fused_batch_ok(p)) return fused_batch_steps(p, psi, nsteps);
   std::vector<Group> groups = make_groups(p);
   cudaStream_t s = p->stream;
-  bool any32 = false;
   for (int g = 0; g < (int)groups.size(); ++g) {
     const Group& G = groups[g];
-    if (G.fp64) {
-      for (int f : G.fields) {
-        gp_status st = plain_steps(p, f, (cpx<double>*)psi[f], nsteps);
-        if (st != GP_OK) return st;
-      }
-      continue;
-    }
-    any32 = true;
     // tables are created before any capture starts
     const FieldPlan& F = p->f[G.fields[0]];
-    if (!ktable(p, G.fields[0], F.prm.dt, false) || !ktable(p, G.fields[0], 0.5 * F.prm.dt, false))
+    if (!ktable(p, G.fields[0], F.prm.dt, G.fp64) || !ktable(p, G.fields[0], 0.5 * F.prm.dt, G.fp64))
       return fail(p, GP_ERR_OOM, "kinetic table allocation");
-    if (plane_on(p, G.n)) {
+    if (!G.fp64 && plane_on(p, G.n)) {
       gp_status st = ensure_plane_sync(p, plane_sync_ints(G.n, (int)G.fields.size()));
       if (st != GP_OK) return st;
     }
   }
-  if (!any32) return GP_OK;
 
   std::vector<Item> pro, cyc, tail, epi;
   for (int g = 0; g < (int)groups.size(); ++g) {
     const Group& G = groups[g];
-    if (G.fp64) continue;
     const double dt = p->f[G.fields[0]].prm.dt, h = 0.5 * dt;
-    const bool pl = plane_on(p, G.n);
+    const bool pl = !G.fp64 && plane_on(p, G.n);
     if (G.split == GP_SPLIT_NKN) {
       pro.push_back({g, 2, OP_N_FWD, h, 0.0});
       k_block(pro, g, dt, pl);
@@ -485,15 +459,15 @@ gp_status step_field(gp_plan* p, int field, void* psi, int nsteps) {
   std::vector<void*> ptrs(p->f.size(), nullptr);
   ptrs[field] = psi;
   FieldPlan& F = p->f[field];
-  if (F.fp64) return plain_steps(p, field, (cpx<double>*)psi, nsteps);
   if (nsteps == 0) return GP_OK;
   Group G;
   G.fields.push_back(field);
   G.n = F.n;
+  G.fp64 = F.fp64;
   G.split = F.prm.split;
   std::vector<Group> groups{G};
   const double dt = F.prm.dt, h = 0.5 * dt;
-  const bool pl = plane_on(p, G.n);
+  const bool pl = !G.fp64 && plane_on(p, G.n);
   if (pl) {
     gp_status st = ensure_plane_sync(p, plane_sync_ints(G.n, 1));
     if (st != GP_OK) return st;

@@ -29,22 +29,14 @@ template <typename T> struct SweepArgs {
   int count;                // number of fields in psi[]
   const tw_t<T>* tw_fwd;    // forward Stockham twiddles for length N
   const tw_t<T>* tw_inv;    // inverse Stockham twiddles for length N
-  const cpx<T>* ek;         // float64: exp(-i alpha s k^2) by grid index, length N (OP_FWD_K_INV)
-  const float4* ekx;        // float32: the same as hi/lo pairs, length N
-  const float4* ek2;        // float32: E[i1] E[i2] / N^3 as hi/lo pairs, index i2 * N + i1
-  KConst k_norm;            // float64: factor applied with K, 1/N^3
+  const float4* ekx;        // exp(-i alpha s k^2) by grid index as hi/lo pairs, length N (OP_FWD_K_INV)
+  const float4* ek2;        // E[i1] E[i2] / N^3 as hi/lo pairs, index i2 * N + i1
   T nl_coef;                // beta * s of N(s)
   T nl_shift;               // c of N(s): 1 (eq-gpe-num) or 0
   int op;
   int axis;                 // 0: x (contiguous rows), 1: y, 2: z (strided pencils)
   int scale_inv;            // 1: inverse ops multiply by 1/N; 0: normalisation done with K
 };
-
-// K factor of one element (float64): E[kx] (E[ky] E[kz]) from the table of exp(-i alpha s k^2), then 1/N^3.
-__device__ __forceinline__ double2 kinetic_apply(double2 x, double2 e_other, double2 e_pos, KConst norm) {
-  const double2 y = cmul(x, cmul(e_pos, e_other));
-  return double2{y.x * norm.v, y.y * norm.v};
-}
 
 template <typename V> __device__ __forceinline__ V kscale(V x, KConst k) { return V{kmul(x.x, k), kmul(x.y, k)}; }
 
@@ -229,17 +221,10 @@ __device__ __forceinline__ void sweep_op_body(const SweepArgs<T>& a, int t, int 
     fft_regs<T, L, B, Lay, false, WARP_X, TW_SH, NB>(v, t, p, sm, lay, a.tw_fwd);
   }
   if constexpr (OP == OP_FWD_K_INV) {
-    if constexpr (sizeof(T) == 4) {
-      // two products by factors exact to float64 (hi + lo), each rounded once: the magnitude
-      // of the field is not biased by the kinetic factor, which is the same for a given k in
-      // every step
+    // two products by factors exact to float64 (hi + lo), each rounded once: the magnitude of the
+    // field is not biased by the kinetic factor, which is the same for a given k in every step
 #pragma unroll
-      for (int e = 0; e < E; ++e) v[e] = twmul_k(twmul_k(v[e], __ldg(a.ekx + out_pos<L, false>(e, t))), eo);
-    } else {
-      const V eo = cmul(__ldg(a.ek + i1), __ldg(a.ek + i2));
-#pragma unroll
-      for (int e = 0; e < E; ++e) v[e] = kinetic_apply(v[e], eo, __ldg(a.ek + out_pos<L, false>(e, t)), a.k_norm);
-    }
+    for (int e = 0; e < E; ++e) v[e] = twmul_k(twmul_k(v[e], __ldg(a.ekx + out_pos<L, false>(e, t))), eo);
     xsync<WARP_X, NB>();
     fft_regs<T, L, B, Lay, true, WARP_X, TW_SH, NB>(v, t, p, sm, lay, a.tw_inv);
   }

@@ -70,6 +70,30 @@ static __global__ void k_reduce_max(const double* __restrict__ part, int nblocks
   }
 }
 
+// out[a] = the sum (a < na) or, for a = na, the maximum over blocks b of part[b * stride + a];
+// one block of 256 threads per quantity, fixed order
+static __global__ void k_reduce_cols(const double* __restrict__ part, int nblocks, int stride, int na,
+                                     double* out) {
+  const int a = blockIdx.x;
+  __shared__ double red[8];
+  double s = 0.0;
+  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
+    const double v = part[(size_t)b * stride + a];
+    s = a < na ? s + v : fmax(s, v);
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double v = __shfl_xor_sync(0xffffffffu, s, o);
+    s = a < na ? s + v : fmax(s, v);
+  }
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int q = 1; q < (int)(blockDim.x >> 5); ++q) s = a < na ? s + red[q] : fmax(s, red[q]);
+    out[a] = s;
+  }
+}
+
 // target = sum / npts (the mean that a renormalisation keeps)
 static __global__ void k_scale_to_mean(const double* sum, double* target, double npts) { *target = *sum / npts; }
 

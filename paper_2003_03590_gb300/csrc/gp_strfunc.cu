@@ -4,8 +4,9 @@
 // with the superfluid velocity v = 2 alpha Im(psi* grad psi) / |psi|^2 (eq-scaling-rhov; the
 // spectral gradient of the diagnostics, Nyquist-zeroed wavenumbers; v = 0 where |psi|^2 < 1e-12).
 //
-// Pipeline: one forward 3D FFT, the three gradient spectra, three inverse FFTs, a pointwise
-// kernel that writes the three real velocity components, then per direction one kernel over
+// Pipeline: the three real velocity components -- float32 fields: one derivative kernel per axis
+// (gp_deriv.cuh) that writes v_j; float64 fields: one forward 3D FFT, the three gradient spectra, three
+// inverse FFTs and a pointwise kernel -- then per direction one kernel over
 // "pencils" (the N points of a line along e_j).  A block stages W pencils in shared memory, each
 // row followed by a wrapped copy of its start so that the periodic shift needs no modulo, and
 // every thread sums R consecutive separations of one pencil at a time: a register window of 2R
@@ -16,8 +17,8 @@
 #include <cmath>
 #include <vector>
 
+#include "gp_deriv.cuh"
 #include "gp_internal.h"
-#include "gp_reduce.cuh"
 
 namespace gp {
 namespace {
@@ -55,6 +56,25 @@ __global__ void k_sf_velocity(const cpx<T>* __restrict__ psi, const cpx<T>* __re
     vy[i] = f * (p.x * b.y - p.y * b.x);
     vz[i] = f * (p.x * c.y - p.y * c.x);
   }
+}
+
+// v_j from d_j psi (one axis, float32)
+template <int AXIS_> struct VelEpi : DerivEpi {
+  static constexpr int AXIS = AXIS_;
+  float* v;
+  float alpha2;
+  __device__ __forceinline__ float2 point(State&, long, float2 p, float2 g, float) const {
+    const float rho = p.x * p.x + p.y * p.y;
+    return float2{(rho >= eps_rho<float>() ? alpha2 / rho : 0.0f) * (p.x * g.y - p.y * g.x), 0.0f};
+  }
+  __device__ __forceinline__ void put(long i, float2 u) const { v[i] = u.x; }
+};
+template <int AXIS> cudaError_t velocity(FieldPlan& F, const float2* psi, float* v, cudaStream_t s) {
+  const DerivArgs a{psi, (const tw_t<float>*)F.t32.tw_fwd, (const tw_t<float>*)F.t32.tw_inv};
+  VelEpi<AXIS> epi;
+  epi.v = v;
+  epi.alpha2 = (float)(2.0 * F.alpha);
+  return deriv(F.n, a, epi, s);
 }
 
 template <typename T, int P> __device__ __forceinline__ T ipow(T d) {
@@ -146,12 +166,23 @@ __global__ void __launch_bounds__(SF_THREADS) k_strfunc(const T* __restrict__ v,
   }
 }
 
-// out[s] = sum over blocks b (in order) of part[b * ns + s]
-__global__ void k_sf_sum_blocks(const double* __restrict__ part, int nblocks, int ns, double* out) {
-  for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < ns; s += gridDim.x * blockDim.x) {
-    double t = 0.0;
-    for (int b = 0; b < nblocks; ++b) t += part[(long long)b * ns + s];
-    out[s] = t;
+// out[j][s] = sum over blocks b of part[j][b * ns + s] in a fixed order: 32 separations per block of
+// 32 x 8 threads, each of the 8 rows adding every 8th block, then the 8 partial sums in turn.  (One
+// thread per separation adding all blocks was a chain of 304 dependent loads: 52 us at 192^3, 3 launches.)
+__global__ void __launch_bounds__(256) k_sf_sum_blocks(const double* __restrict__ part, int nblocks, int ns, double* out) {
+  __shared__ double red[8][32];
+  const int s = blockIdx.x * 32 + (threadIdx.x & 31), r = threadIdx.x >> 5;
+  const double* q = part + (long long)blockIdx.y * nblocks * ns;
+  double t = 0.0;
+  if (s < ns) {
+#pragma unroll 4
+    for (int b = r; b < nblocks; b += 8) t += q[(long long)b * ns + s];
+  }
+  red[r][threadIdx.x & 31] = t;
+  __syncthreads();
+  if (r == 0 && s < ns) {
+    for (int k = 1; k < 8; ++k) t += red[k][threadIdx.x & 31];
+    out[(long long)blockIdx.y * ns + s] = t;
   }
 }
 
@@ -208,7 +239,7 @@ gp_status strfunc_impl(gp_plan* p, int field, const cpx<T>* psi, int order, doub
   const int ntiles = n * n / W;
   const int nblocks = ntiles < 2 * 152 ? ntiles : 2 * 152;
   const size_t vz_bytes = ((size_t)npts * sizeof(T) + 255) / 256 * 256;
-  gp_status st = ensure_ws(p, field, 4 * fb + vz_bytes + ((size_t)nblocks * ns + 3 * ns) * sizeof(double));
+  gp_status st = ensure_ws(p, field, 4 * fb + vz_bytes + ((size_t)3 * nblocks * ns + 3 * ns) * sizeof(double));
   if (st != GP_OK) return st;
   cpx<T>* w0 = (cpx<T>*)F.ws;
   cpx<T>* w1 = w0 + npts;
@@ -218,30 +249,26 @@ gp_status strfunc_impl(gp_plan* p, int field, const cpx<T>* psi, int order, doub
   T* vy = vx + npts;
   T* vz = (T*)(w3 + npts);
   double* part = (double*)((unsigned char*)vz + vz_bytes);
-  double* sums = part + (size_t)nblocks * ns;
-  GP_CUDA(p, cudaMemcpyAsync(w0, psi, fb, cudaMemcpyDeviceToDevice, s));
-  cpx<T>* all[4] = {w0, w1, w2, w3};
-  auto transform = [&](int first, int count, bool inverse) -> cudaError_t {
-    if constexpr (sizeof(T) == 4) return fft3_many(p, F, all + first, count, inverse, s);
-    for (int k = first; k < first + count; ++k) {
-      cudaError_t e = fft3<T>(F, all[k], inverse, s);
-      if (e != cudaSuccess) return e;
-    }
-    return cudaSuccess;
-  };
-  GP_CUDA(p, transform(0, 1, false));
-  const unsigned g = sf_grid(npts);
-  k_sf_grad<T><<<g, 256, 0, s>>>(w0, w1, w2, w3, n);
-  GP_CUDA(p, cudaGetLastError());
-  GP_CUDA(p, transform(1, 3, true));
-  k_sf_velocity<T><<<g, 256, 0, s>>>(psi, w1, w2, w3, vx, vy, vz, npts, F.alpha);
-  GP_CUDA(p, cudaGetLastError());
-  const T* comp[3] = {vx, vy, vz};
-  for (int j = 0; j < 3; ++j) {
-    GP_CUDA(p, strfunc_order<T>(order, comp[j], n, j, part, nblocks, s));
-    k_sf_sum_blocks<<<(ns + 127) / 128, 128, 0, s>>>(part, nblocks, ns, sums + (size_t)j * ns);
+  double* sums = part + (size_t)3 * nblocks * ns;
+  if constexpr (sizeof(T) == 4) {
+    GP_CUDA(p, velocity<0>(F, psi, vx, s));
+    GP_CUDA(p, velocity<1>(F, psi, vy, s));
+    GP_CUDA(p, velocity<2>(F, psi, vz, s));
+  } else {
+    GP_CUDA(p, cudaMemcpyAsync(w0, psi, fb, cudaMemcpyDeviceToDevice, s));
+    cpx<T>* all[4] = {w0, w1, w2, w3};
+    GP_CUDA(p, fft3<T>(F, w0, false, s));
+    const unsigned g = sf_grid(npts);
+    k_sf_grad<T><<<g, 256, 0, s>>>(w0, w1, w2, w3, n);
+    GP_CUDA(p, cudaGetLastError());
+    for (int k = 1; k < 4; ++k) GP_CUDA(p, fft3<T>(F, all[k], true, s));
+    k_sf_velocity<T><<<g, 256, 0, s>>>(psi, w1, w2, w3, vx, vy, vz, npts, F.alpha);
     GP_CUDA(p, cudaGetLastError());
   }
+  const T* comp[3] = {vx, vy, vz};
+  for (int j = 0; j < 3; ++j) GP_CUDA(p, strfunc_order<T>(order, comp[j], n, j, part + (size_t)j * nblocks * ns, nblocks, s));
+  k_sf_sum_blocks<<<dim3((ns + 31) / 32, 3), 256, 0, s>>>(part, nblocks, ns, sums);
+  GP_CUDA(p, cudaGetLastError());
   std::vector<double> h((size_t)3 * ns);
   GP_CUDA(p, cudaMemcpyAsync(h.data(), sums, h.size() * sizeof(double), cudaMemcpyDeviceToHost, s));
   GP_CUDA(p, cudaStreamSynchronize(s));

@@ -236,8 +236,9 @@ long long gp_launch_count(const gp_plan* plan);
  * separate sweeps with their own variants.  cache_path (NULL: none) names a JSON file of earlier
  * choices keyed by GPU name, length, axis and op; cached choices are reused without timing and
  * new ones are added.  Synchronises the stream and drops captured graphs.
- * gp_plan_sweep_variant returns the variant in use for a kind (default 0: fused plane kernel
- * and TMA sweeps wherever the length has them).  gp_plan_set_sweep_variant sets it by hand
+ * gp_plan_sweep_variant returns the variant chosen for a kind by the tuner or by hand (0 if none
+ * was: the library then uses, per length, the kernel measured fastest; 2 for lengths without TMA
+ * kernels).  gp_plan_set_sweep_variant sets it by hand, 0 included
  * (GP_ERR_INVALID_ARG for an unknown kind or variant); it synchronises the stream and drops
  * captured graphs. */
 gp_status gp_plan_autotune(gp_plan* plan, const char* cache_path);

@@ -140,7 +140,8 @@ template <typename T> cudaError_t launch_vjp_nonlinear(const cpx<T>* psi_in, cpx
 // stages, 4 TMA with another split into stages and compute groups (lengths >= 512); for OP_PLANE 0 means the fused
 // plane kernel, 3 the same with two stages and 2 the three separate sweeps it replaces
 enum { VARIANT_TMA = 0, VARIANT_TMA_ONE = 1, VARIANT_PLAIN = 2, VARIANT_TMA_2STAGE = 3, VARIANT_TMA_GROUPS = 4 };
-int sweep_variant(gp_plan* p, int n, int axis, int op);
+int sweep_variant(gp_plan* p, int n, int axis, int op);    // as reported: the plan's choice, or 0
+int kernel_variant(gp_plan* p, int n, int axis, int op);   // as launched: the plan's choice, or the length's
 bool plane_on(gp_plan* p, int n);
 gp_status ensure_plane_sync(gp_plan* p, size_t ints);
 // one float32 sweep of the given kind with the given variant (used by the autotuner)

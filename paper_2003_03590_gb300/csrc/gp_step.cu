@@ -34,9 +34,36 @@ int sweep_variant(gp_plan* p, int n, int axis, int op) {
   return VARIANT_TMA;
 }
 
+// The kernel of a sweep kind when none was chosen for the plan, by the length.  Measured on GB300, us per
+// launch of one field (the batched steps order the same way):
+//   y, x, y as the fused plane kernel / as three sweeps: 32^3 27 / 13, 64^3 30 / 15, 96^3 39 / 26, 128^3
+//     39 / 31, 192^3 113 / 92, 256^3 144 / 156, 512^3 1655 / 1260, 1024^3 12800 / 10300: fused where its
+//     planes both fill the GPU and are few enough to stay in L2, which is 256;
+//   x sweeps (forward, K, inverse), TMA / one tile per CTA: 128^3 16.9 / 14.8, 192^3 55 / 52, 256^3 71 / 66,
+//     512^3 577 / 530, 1024^3 5510 / 5005: rows are contiguous, direct loads lose nothing;
+//   y and z up to 128 points: one step of 24 fields of 64^3 75 us with TMA kernels, 69 without, of 16 fields
+//     of 96^3 251 / 242, of 8 fields of 128^3 220 / 203 (a CTA has few tiles to pipeline); at 192 two
+//     stages: z inverse-N-forward 45.6 / 37.8 / 37.3 (three stages / one tile per CTA / two stages);
+//   z at 1024 with one transform: 6840 / 5000 (128-byte rows without the stages for them).
+static int default_variant(int n, int axis, int op) {
+  if (op == OP_PLANE) return n == 256 ? VARIANT_TMA : VARIANT_PLAIN;
+  if (axis == 0 || n <= 128) return VARIANT_PLAIN;
+  if (n == 192) return VARIANT_TMA_2STAGE;
+  if (n == 1024 && axis == 2 && op != OP_INV_N_FWD) return VARIANT_PLAIN;
+  return VARIANT_TMA;
+}
+int kernel_variant(gp_plan* p, int n, int axis, int op) {
+  if (!p->use_tma || !tma_supported(n)) return VARIANT_PLAIN;
+  const long long k = tune_key(n, axis, op);
+  for (const auto& e : p->tune)
+    if (e.first == k) return e.second;
+  if (op == OP_PLANE && p->plane_skip > 0) return VARIANT_TMA;   // gp_plan_test_timeout tests the fused kernel
+  return default_variant(n, axis, op);
+}
+
 // forward y, x (forward, K, inverse) and inverse y of a step as one fused plane-kernel launch
 bool plane_on(gp_plan* p, int n) {
-  const int v = sweep_variant(p, n, 1, OP_PLANE);
+  const int v = kernel_variant(p, n, 1, OP_PLANE);
   return v == VARIANT_TMA || v == VARIANT_TMA_ONE || v == VARIANT_TMA_2STAGE || v == VARIANT_TMA_GROUPS;
 }
 
@@ -83,7 +110,7 @@ cudaError_t launch_sweep_variant(gp_plan* p, int n, const SweepArgs<float>& a, v
     for (const auto& o : ops) {
       b.axis = o[0];
       b.op = o[1];
-      cudaError_t e = launch_sweep_variant(p, n, b, psi, sweep_variant(p, n, b.axis, b.op), s);
+      cudaError_t e = launch_sweep_variant(p, n, b, psi, kernel_variant(p, n, b.axis, b.op), s);
       if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -105,7 +132,7 @@ cudaError_t fft1_many(gp_plan* p, FieldPlan& F, cpx<float>* const* xs, int count
   a.op = inverse ? OP_INV : OP_FWD;
   a.scale_inv = 1;
   a.axis = axis;
-  return launch_sweep_variant(p, F.n, a, ptrs, sweep_variant(p, F.n, a.axis, a.op), s);
+  return launch_sweep_variant(p, F.n, a, ptrs, kernel_variant(p, F.n, a.axis, a.op), s);
 }
 // 3D transforms of `count` float32 fields of one plan length, one launch per axis for all of
 // them, through the kernel variants chosen for the forward and inverse y/z sweeps (x: TMA)
@@ -199,7 +226,7 @@ gp_status launch_item(gp_plan* p, const Group& G, const Item& it, void* const* p
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (p->prof) {
     static const char* opn[] = {"", "fwd", "inv", "inv_n_fwd", "n_fwd", "inv_n", "fwd_k_inv", "fwd_k_inv"};
-    const bool tma = sweep_variant(p, G.n, it.axis, it.op) != VARIANT_PLAIN;
+    const bool tma = kernel_variant(p, G.n, it.axis, it.op) != VARIANT_PLAIN;
     std::string name = it.op == OP_PLANE ? std::string("k_tma_plane<") + std::to_string(G.n) + ">:y_fwd_x_fwd_k_inv_y_inv:xy"
                        : std::string(tma ? (G.n >= 256 && !(G.n == 512 && it.axis == 1) ? "k_warp_sweep<"
                                             : it.axis == 0 ? "k_tma_contig<" : "k_tma_strided<")
@@ -222,7 +249,7 @@ gp_status launch_item(gp_plan* p, const Group& G, const Item& it, void* const* p
   }
   void* ptrs[GP_MAXB];
   for (int k = 0; k < a.count; ++k) ptrs[k] = psi[G.fields[k]];
-  cudaError_t e = launch_sweep_variant(p, G.n, a, ptrs, sweep_variant(p, G.n, it.axis, it.op), s);
+  cudaError_t e = launch_sweep_variant(p, G.n, a, ptrs, kernel_variant(p, G.n, it.axis, it.op), s);
   if (e != cudaSuccess) return cuda_fail(p, e, "sweep launch");
   if (p->prof) GP_CUDA(p, cudaEventRecord(e1, s));
   p->launches += 1;

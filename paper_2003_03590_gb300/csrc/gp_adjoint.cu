@@ -179,11 +179,213 @@ template <typename T> static gp_status ekin_grad_impl(gp_plan* p, int field, con
   return GP_OK;
 }
 
-template <typename T> static gp_status adjoint_impl(gp_plan* p, int field, const cpx<T>* psi_n, cpx<T>* lam, int nsteps) {
+// ---------------------------------------------------------------- float32 segments
+// The z sweeps of a segment, each one pass over its fields (gp_sweep.cuh's tiles and transforms):
+//   Z_STATE  [inverse z], N(c1), write the state to `out`, N(c2), [forward z], write back to dst
+//   Z_VJP    [inverse z], the cotangent through N(c2) at its input S, then through N(c1) at its output S
+//            (c = 0: skipped), [forward z]
+// At a state S between two steps the cotangent passes the opening N of one step and the closing N of the
+// step before; both have |psi| = |S|, and with psi_out = S the closing one is
+//   VJP_N lam = exp(+i phi) (lam + 2 coef Im(conj(lam) S) S),
+// so that only the states between the steps are needed.  A step back is then one z sweep and the sweeps
+// of K(-dt); the states come from one z sweep and the sweeps of K(dt) each.  (With N, K and every
+// sub-flow's input recomputed by kernels of their own a step took 18 launches; GB300, 128^3: 0.25 ms per
+// step, now 0.14 ms, forward run included.)
+// |phase| > 1/2 is rare (see nonlinear_large)
+static __device__ __noinline__ float2 sincos_large(float ph) {
+  float sn, cs;
+  sincosf(ph, &sn, &cs);
+  return float2{cs, sn};
+}
+__device__ __forceinline__ float2 phase_factor(float ph) {   // (cos, sin)
+  if (fabsf(ph) <= 0.5f) {
+    float sn, cm1;
+    sincos_m1_small(ph, &sn, &cm1);
+    return float2{1.0f + cm1, sn};
+  }
+  return sincos_large(ph);
+}
+
+enum { Z_STATE = 0, Z_VJP = 1 };
+struct AdjZ {
+  const float2* src;      // read
+  float2* dst;            // written (may be src)
+  const float2* state;    // Z_VJP: S
+  float2* out;            // Z_STATE: the state between N(c1) and N(c2), or null
+  const tw_t<float>* tw_fwd;
+  const tw_t<float>* tw_inv;
+  float c1, c2, shift;
+};
+template <int L, int WHAT, bool INV, bool FWD> __device__ __forceinline__ void adj_z_tile(const AdjZ& a) {
+  constexpr int E = Plan<L>::E, B = strided_batch<float, L>();
+  extern __shared__ __align__(16) unsigned char smraw[];
+  float2* sm = reinterpret_cast<float2*>(smraw);
+  const int p = threadIdx.x % B, t = threadIdx.x / B;
+  const int tile = blockIdx.x;
+  const long base = (tile % (L / B)) * B + p + (long)(tile / (L / B)) * L, st = (long)L * L;
+  LayStrided lay{B};
+  float2 v[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) v[e] = a.src[base + in_pos<L, INV>(e, t) * st];
+  if constexpr (INV) fft_regs<float, L, B, LayStrided, true>(v, t, p, sm, lay, a.tw_inv);
+  if constexpr (WHAT == Z_STATE) {
+    if (a.c1 != 0.0f) nonlinear_all<E>(v, a.c1, a.shift);
+    if (a.out) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) a.out[base + in_pos<L, false>(e, t) * st] = v[e];
+    }
+    if (a.c2 != 0.0f) nonlinear_all<E>(v, a.c2, a.shift);
+  } else if (a.c1 != 0.0f || a.c2 != 0.0f) {
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const float2 S = a.state[base + in_pos<L, false>(e, t) * st];
+      const float r = S.x * S.x + S.y * S.y - a.shift;
+      float2 l = v[e];
+      float2 w;
+      if (a.c2 != 0.0f) {
+        w = phase_factor(a.c2 * r);
+        const float2 po{S.x * w.x + S.y * w.y, S.y * w.x - S.x * w.y};          // exp(-i phi) S
+        const float g = 2.0f * a.c2 * (l.x * po.y - l.y * po.x);
+        l = float2{l.x * w.x - l.y * w.y + g * S.x, l.y * w.x + l.x * w.y + g * S.y};
+      }
+      if (a.c1 != 0.0f) {
+        if (a.c1 != a.c2) w = phase_factor(a.c1 * r);
+        const float g = 2.0f * a.c1 * (l.x * S.y - l.y * S.x);
+        const float2 m{l.x + g * S.x, l.y + g * S.y};
+        l = float2{m.x * w.x - m.y * w.y, m.y * w.x + m.x * w.y};
+      }
+      v[e] = l;
+    }
+  }
+  if constexpr (FWD) {
+    if constexpr (INV) __syncthreads();   // the first transform's exchanges
+    fft_regs<float, L, B, LayStrided, false>(v, t, p, sm, lay, a.tw_fwd);
+  }
+#pragma unroll
+  for (int e = 0; e < E; ++e) a.dst[base + (FWD ? out_pos<L, false>(e, t) : in_pos<L, false>(e, t)) * st] = v[e];
+}
+template <int L, int WHAT, bool INV, bool FWD>
+__global__ void __launch_bounds__(strided_batch<float, L>() * (L / Plan<L>::E)) k_adj_z(const AdjZ a) {
+  adj_z_tile<L, WHAT, INV, FWD>(a);
+}
+template <int L, int WHAT, bool INV, bool FWD>
+__global__ void __launch_bounds__(strided_batch<float, L>() * (L / Plan<L>::E), rcap_blocks<float, L>(false)) k_adj_z_rc(const AdjZ a) {
+  adj_z_tile<L, WHAT, INV, FWD>(a);
+}
+template <int L, int WHAT, bool INV, bool FWD> static cudaError_t adj_z_launch(const AdjZ& a, cudaStream_t s) {
+  constexpr int B = strided_batch<float, L>(), NT = B * (L / Plan<L>::E);
+  constexpr size_t smem = sizeof(float2) * (size_t)L * B;
+  constexpr auto kern = [] {
+    if constexpr (rcapped<float, L>()) return k_adj_z_rc<L, WHAT, INV, FWD>;
+    else return k_adj_z<L, WHAT, INV, FWD>;
+  }();
+  static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (attr != cudaSuccess) return attr;
+  kern<<<(L / B) * L, NT, smem, s>>>(a);
+  return cudaGetLastError();
+}
+template <int WHAT, bool INV, bool FWD> static cudaError_t adj_z(int n, const AdjZ& a, cudaStream_t s) {
+  switch (n) {
+#define GP_CASE(L) case L: return adj_z_launch<L, WHAT, INV, FWD>(a, s);
+    GP_SIZES(GP_CASE)
+#undef GP_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+#define GP_K(x, t)                                    \
+  do {                                                \
+    gp_status st_ = kinetic_block(p, field, (x), (t)); \
+    if (st_ != GP_OK) return st_;                     \
+  } while (0)
+static gp_status adjoint_f32(gp_plan* p, int field, const float2* psi_n, float2* lam, int nsteps) {
   FieldPlan& F = p->f[field];
   const long long npts = F.npts;
   cudaStream_t s = p->stream;
-  const size_t fb = (size_t)npts * sizeof(cpx<T>);
+  // the work field and nsteps - 1 states; a copy of psi_n where lam, written from the first sweep back on, overlaps it
+  const bool overlap = psi_n < lam + npts && lam < psi_n + npts;
+  const size_t need = (size_t)(nsteps + overlap) * (size_t)npts * sizeof(float2);
+  if (p->adj_bytes < need) {
+    if (p->adj_ws) cudaFree(p->adj_ws);
+    p->adj_ws = nullptr;
+    p->adj_bytes = 0;
+    GP_CUDA(p, cudaMalloc(&p->adj_ws, need));
+    p->adj_bytes = need;
+  }
+  float2* work = (float2*)p->adj_ws;
+  auto state = [&](int m) { return work + (size_t)m * npts; };         // m = 1 .. nsteps - 1
+  if (overlap) {
+    GP_CUDA(p, cudaMemcpyAsync(state(nsteps), psi_n, (size_t)npts * sizeof(float2), cudaMemcpyDeviceToDevice, s));
+    psi_n = state(nsteps);
+  }
+  const double dt = F.prm.dt, h = 0.5 * dt;
+  const float ch = (float)(F.beta * h), cd = (float)(F.beta * dt), shift = F.prm.nonlin_minus_one ? 1.0f : 0.0f;
+  AdjZ z{};
+  z.tw_fwd = (const tw_t<float>*)F.t32.tw_fwd;
+  z.tw_inv = (const tw_t<float>*)F.t32.tw_inv;
+  z.shift = shift;
+  auto flow = [&](const float2* src, float2* dst, float2* out, float c1, float c2) {
+    z.src = src, z.dst = dst, z.out = out, z.state = nullptr, z.c1 = c1, z.c2 = c2;
+  };
+  auto vjp = [&](const float2* S, float c1, float c2) { z.src = z.dst = lam, z.out = nullptr, z.state = S, z.c1 = c1, z.c2 = c2; };
+  if (F.prm.split == GP_SPLIT_NKN) {
+    // states S_1 .. S_{n-1} into their slots, S_n into work
+    flow(psi_n, work, nullptr, 0.0f, ch);
+    GP_CUDA(p, (adj_z<Z_STATE, false, true>(F.n, z, s)));
+    for (int m = 1; m <= nsteps; ++m) {
+      GP_K(work, dt);
+      if (m < nsteps) {
+        flow(work, work, state(m), ch, ch);
+        GP_CUDA(p, (adj_z<Z_STATE, true, true>(F.n, z, s)));
+      } else {
+        flow(work, work, nullptr, ch, 0.0f);
+        GP_CUDA(p, (adj_z<Z_STATE, true, false>(F.n, z, s)));
+      }
+    }
+    vjp(work, ch, 0.0f);
+    GP_CUDA(p, (adj_z<Z_VJP, false, true>(F.n, z, s)));
+    for (int m = nsteps - 1; m >= 0; --m) {
+      GP_K(lam, -dt);
+      if (m > 0) {
+        vjp(state(m), ch, ch);
+        GP_CUDA(p, (adj_z<Z_VJP, true, true>(F.n, z, s)));
+      } else {
+        vjp(psi_n, 0.0f, ch);
+        GP_CUDA(p, (adj_z<Z_VJP, true, false>(F.n, z, s)));
+      }
+    }
+  } else {
+    // the inputs a_m of N(dt): a_0 .. a_{n-2} into slots 1 .. n-1, a_{n-1} into work
+    flow(psi_n, work, nullptr, 0.0f, 0.0f);
+    GP_CUDA(p, (adj_z<Z_STATE, false, true>(F.n, z, s)));
+    GP_K(work, h);
+    for (int m = 0; m < nsteps - 1; ++m) {
+      flow(work, work, state(m + 1), 0.0f, cd);
+      GP_CUDA(p, (adj_z<Z_STATE, true, true>(F.n, z, s)));
+      GP_K(work, dt);
+    }
+    flow(work, work, nullptr, 0.0f, 0.0f);
+    GP_CUDA(p, (adj_z<Z_STATE, true, false>(F.n, z, s)));
+    vjp(nullptr, 0.0f, 0.0f);
+    GP_CUDA(p, (adj_z<Z_VJP, false, true>(F.n, z, s)));
+    GP_K(lam, -h);
+    for (int m = nsteps - 1; m >= 0; --m) {
+      vjp(m == nsteps - 1 ? work : state(m + 1), 0.0f, cd);
+      GP_CUDA(p, (adj_z<Z_VJP, true, true>(F.n, z, s)));
+      GP_K(lam, m > 0 ? -dt : -h);
+    }
+    vjp(nullptr, 0.0f, 0.0f);
+    GP_CUDA(p, (adj_z<Z_VJP, true, false>(F.n, z, s)));
+  }
+  return GP_OK;
+}
+#undef GP_K
+
+static gp_status adjoint_f64(gp_plan* p, int field, const double2* psi_n, double2* lam, int nsteps) {
+  FieldPlan& F = p->f[field];
+  const long long npts = F.npts;
+  cudaStream_t s = p->stream;
+  const size_t fb = (size_t)npts * sizeof(double2);
   const size_t need = (size_t)(nsteps + 1) * fb;
   if (p->adj_bytes < need) {
     if (p->adj_ws) cudaFree(p->adj_ws);
@@ -192,14 +394,13 @@ template <typename T> static gp_status adjoint_impl(gp_plan* p, int field, const
     GP_CUDA(p, cudaMalloc(&p->adj_ws, need));
     p->adj_bytes = need;
   }
-  cpx<T>* S = (cpx<T>*)p->adj_ws;
-  cpx<T>* tmp = S + (size_t)nsteps * npts;
+  double2* S = (double2*)p->adj_ws;
+  double2* tmp = S + (size_t)nsteps * npts;
   const double dt = F.prm.dt, h = 0.5 * dt, shift = F.prm.nonlin_minus_one ? 1.0 : 0.0;
-  const bool f64 = sizeof(T) == 8;
-  const void* kd = ktable(p, field, dt, f64);
-  const void* kmd = ktable(p, field, -dt, f64);
-  const void* kh = ktable(p, field, h, f64);
-  const void* kmh = ktable(p, field, -h, f64);
+  const void* kd = ktable(p, field, dt, true);
+  const void* kmd = ktable(p, field, -dt, true);
+  const void* kh = ktable(p, field, h, true);
+  const void* kmh = ktable(p, field, -h, true);
   if (!kd || !kmd || !kh || !kmh) return fail(p, GP_ERR_OOM, "kinetic table allocation");
   // recompute the states at the start of every step of the segment
   GP_CUDA(p, cudaMemcpyAsync(S, psi_n, fb, cudaMemcpyDeviceToDevice, s));
@@ -209,19 +410,19 @@ template <typename T> static gp_status adjoint_impl(gp_plan* p, int field, const
     if (st != GP_OK) return st;
   }
   for (int m = nsteps - 1; m >= 0; --m) {
-    const cpx<T>* Sm = S + (size_t)m * npts;
+    const double2* Sm = S + (size_t)m * npts;
     GP_CUDA(p, cudaMemcpyAsync(tmp, Sm, fb, cudaMemcpyDeviceToDevice, s));
     if (F.prm.split == GP_SPLIT_NKN) {
-      GP_CUDA(p, launch_nonlinear<T>(tmp, npts, F.beta * h, shift, s));          // a = N(h) S_m
-      GP_CUDA(p, kinetic3<T>(F, tmp, kd, s));                                    // b = K(dt) a
-      GP_CUDA(p, launch_vjp_nonlinear<T>(tmp, lam, npts, F.beta * h, shift, s)); // through N(h) at b
-      GP_CUDA(p, kinetic3<T>(F, lam, kmd, s));                                   // through K(dt)
-      GP_CUDA(p, launch_vjp_nonlinear<T>(Sm, lam, npts, F.beta * h, shift, s));  // through N(h) at S_m
+      GP_CUDA(p, launch_nonlinear(tmp, npts, F.beta * h, shift, s));          // a = N(h) S_m
+      GP_CUDA(p, kinetic3_f64(F, tmp, kd, s));                                // b = K(dt) a
+      GP_CUDA(p, launch_vjp_nonlinear(tmp, lam, npts, F.beta * h, shift, s)); // through N(h) at b
+      GP_CUDA(p, kinetic3_f64(F, lam, kmd, s));                               // through K(dt)
+      GP_CUDA(p, launch_vjp_nonlinear(Sm, lam, npts, F.beta * h, shift, s));  // through N(h) at S_m
     } else {
-      GP_CUDA(p, kinetic3<T>(F, tmp, kh, s));                                    // a = K(h) S_m
-      GP_CUDA(p, kinetic3<T>(F, lam, kmh, s));                                   // through the last K(h)
-      GP_CUDA(p, launch_vjp_nonlinear<T>(tmp, lam, npts, F.beta * dt, shift, s));// through N(dt) at a
-      GP_CUDA(p, kinetic3<T>(F, lam, kmh, s));                                   // through the first K(h)
+      GP_CUDA(p, kinetic3_f64(F, tmp, kh, s));                                    // a = K(h) S_m
+      GP_CUDA(p, kinetic3_f64(F, lam, kmh, s));                                   // through the last K(h)
+      GP_CUDA(p, launch_vjp_nonlinear(tmp, lam, npts, F.beta * dt, shift, s));// through N(dt) at a
+      GP_CUDA(p, kinetic3_f64(F, lam, kmh, s));                                   // through the first K(h)
     }
   }
   return GP_OK;
@@ -240,8 +441,8 @@ gp_status gp_adjoint_step(gp_plan* p, int field, const void* psi_n, void* lambda
     return fail(p, GP_ERR_INVALID_ARG, "gp_adjoint_step: pointer");
   if (nsteps < 0) return fail(p, GP_ERR_INVALID_ARG, "gp_adjoint_step: negative nsteps");
   if (nsteps == 0) return GP_OK;
-  if (p->f[field].fp64) return adjoint_impl<double>(p, field, (const cpx<double>*)psi_n, (cpx<double>*)lambda, nsteps);
-  return adjoint_impl<float>(p, field, (const cpx<float>*)psi_n, (cpx<float>*)lambda, nsteps);
+  if (p->f[field].fp64) return adjoint_f64(p, field, (const double2*)psi_n, (double2*)lambda, nsteps);
+  return adjoint_f32(p, field, (const float2*)psi_n, (float2*)lambda, nsteps);
 }
 
 gp_status gp_ekin_i_grad(gp_plan* p, int field, const void* psi, void* lambda_out, double eps, double* J_out) {

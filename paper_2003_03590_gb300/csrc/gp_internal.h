@@ -125,16 +125,15 @@ gp_status ensure_ws(gp_plan* p, int field, size_t bytes);
 
 // 3D transforms of a whole field through the pencil sweeps (unfused).
 template <typename T> cudaError_t fft3(FieldPlan& F, cpx<T>* x, bool inverse, cudaStream_t s);
-// K with fused sweeps: fwd z, fwd y, [fwd x, K (table ek), 1/N^3, inv x], inv y, inv z.
+// K of a float64 field with fused sweeps: fwd z, fwd y, [fwd x, K (table ek), 1/N^3, inv x], inv y, inv z.
 // ek: the table that ktable returns
-template <typename T> cudaError_t kinetic3(FieldPlan& F, cpx<T>* x, const void* ek, cudaStream_t s);
+cudaError_t kinetic3_f64(FieldPlan& F, double2* x, const void* ek, cudaStream_t s);
 // the tables of a float64 field's sweeps (ek: from ktable, or null)
 FixArgs fix_args(FieldPlan& F, const void* ek);
 
 // pointwise kernels (gp_pointwise.cu)
-template <typename T> cudaError_t launch_nonlinear(cpx<T>* psi, long long npts, double coef, double shift, cudaStream_t s);
-template <typename T> cudaError_t launch_vjp_nonlinear(const cpx<T>* psi_in, cpx<T>* lam, long long npts, double coef,
-                                                       double shift, cudaStream_t s);
+cudaError_t launch_nonlinear(double2* psi, long long npts, double coef, double shift, cudaStream_t s);
+cudaError_t launch_vjp_nonlinear(const double2* psi_in, double2* lam, long long npts, double coef, double shift, cudaStream_t s);
 
 // sweep variants (gp_step.cu): 0 TMA persistent, 1 TMA one CTA per SM, 2 plain, 3 TMA with two
 // stages, 4 TMA with another split into stages and compute groups (lengths >= 512); for OP_PLANE 0 means the fused
@@ -154,5 +153,7 @@ cudaError_t fft3_many(gp_plan* p, FieldPlan& F, cpx<float>* const* xs, int count
 
 // the time step (gp_step.cu): advance one field by nsteps on the plan's stream
 gp_status step_field(gp_plan* p, int field, void* psi, int nsteps);
+// K(sk) with 1/N^3 on a field in the step's mixed representation (physical along x and y, Fourier along z)
+gp_status kinetic_block(gp_plan* p, int field, void* psi, double sk);
 
 }  // namespace gp

@@ -276,22 +276,20 @@ FixArgs fix_args(FieldPlan& F, const void* ek) {
   a.ek = (const ufix2*)ek;
   return a;
 }
-static SweepArgs<float> f32_args(FieldPlan& F, const void* ek) {
-  SweepArgs<float> a{};
-  a.count = 1;
-  a.tw_fwd = (const tw_t<float>*)F.t32.tw_fwd;
-  a.tw_inv = (const tw_t<float>*)F.t32.tw_inv;
-  a.ekx = (const float4*)ek;
-  if (ek) a.ek2 = (const float4*)ek + F.n;
-  return a;
-}
-template <typename T> static auto sweep_args(FieldPlan& F, const void* ek) {
-  if constexpr (sizeof(T) == 4) return f32_args(F, ek);
-  else return fix_args(F, ek);
+template <typename T> static auto transform_args(FieldPlan& F) {
+  if constexpr (sizeof(T) == 4) {
+    SweepArgs<float> a{};
+    a.count = 1;
+    a.tw_fwd = (const tw_t<float>*)F.t32.tw_fwd;
+    a.tw_inv = (const tw_t<float>*)F.t32.tw_inv;
+    return a;
+  } else {
+    return fix_args(F, nullptr);
+  }
 }
 
 template <typename T> cudaError_t fft3(FieldPlan& F, cpx<T>* x, bool inverse, cudaStream_t s) {
-  auto a = sweep_args<T>(F, nullptr);
+  auto a = transform_args<T>(F);
   a.psi[0] = x;
   a.op = inverse ? OP_INV : OP_FWD;
   a.scale_inv = 1;
@@ -306,8 +304,8 @@ template <typename T> cudaError_t fft3(FieldPlan& F, cpx<T>* x, bool inverse, cu
 template cudaError_t fft3<float>(FieldPlan&, cpx<float>*, bool, cudaStream_t);
 template cudaError_t fft3<double>(FieldPlan&, cpx<double>*, bool, cudaStream_t);
 
-template <typename T> cudaError_t kinetic3(FieldPlan& F, cpx<T>* x, const void* ek, cudaStream_t s) {
-  auto a = sweep_args<T>(F, ek);
+cudaError_t kinetic3_f64(FieldPlan& F, double2* x, const void* ek, cudaStream_t s) {
+  FixArgs a = fix_args(F, ek);
   a.psi[0] = x;
   a.scale_inv = 0;
   const int axes[5] = {2, 1, 0, 1, 2};
@@ -320,8 +318,6 @@ template <typename T> cudaError_t kinetic3(FieldPlan& F, cpx<T>* x, const void* 
   }
   return cudaSuccess;
 }
-template cudaError_t kinetic3<float>(FieldPlan&, cpx<float>*, const void*, cudaStream_t);
-template cudaError_t kinetic3<double>(FieldPlan&, cpx<double>*, const void*, cudaStream_t);
 
 static void free_field(FieldPlan& F) {
   void* ptrs[] = {F.t32.tw_fwd, F.t32.tw_inv, F.t64.tw_fwd, F.t64.tw_inv, F.t64.dir, F.host_buf, F.ws};

@@ -1,4 +1,4 @@
-// gp_pointwise.cu -- pointwise kernels of the plain (unfused) path and of the adjoint.
+// gp_pointwise.cu -- pointwise kernels: the sub-flows of the float64 adjoint, psi from a phase and its gradient.
 #include "gp_internal.h"
 
 namespace gp {
@@ -9,25 +9,23 @@ static inline unsigned grid_for(long long n, int threads) {
 }
 
 // N(s): psi <- exp(-i coef (|psi|^2 - shift)) psi   (Sec. 4.3, exact nonlinear flow)
-template <typename T> __global__ void k_nonlinear(cpx<T>* psi, long long npts, T coef, T shift) {
+__global__ void k_nonlinear(double2* psi, long long npts, double coef, double shift) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < npts; i += (long long)gridDim.x * blockDim.x)
     psi[i] = nonlinear(psi[i], coef, shift);
 }
 
 // VJP of N(s) at input psi_in: lam <- exp(+i phi) lam + 2 coef Im(conj(lam) psi_out) psi_in,
 // phi = coef (|psi_in|^2 - shift), psi_out = exp(-i phi) psi_in, coef = beta s.
-template <typename T>
-__global__ void k_vjp_nonlinear(const cpx<T>* __restrict__ psi_in, cpx<T>* lam, long long npts, T coef, T shift) {
+__global__ void k_vjp_nonlinear(const double2* __restrict__ psi_in, double2* lam, long long npts, double coef, double shift) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < npts; i += (long long)gridDim.x * blockDim.x) {
-    cpx<T> p = psi_in[i], l = lam[i];
-    T ph = coef * (p.x * p.x + p.y * p.y - shift);
-    T sn, cs;
-    if constexpr (sizeof(T) == 4) sincosf(ph, &sn, &cs);
-    else sincos(ph, &sn, &cs);
-    cpx<T> po{p.x * cs + p.y * sn, p.y * cs - p.x * sn};          // exp(-i ph) p
-    T im = l.x * po.y - l.y * po.x;                                 // Im(conj(l) po)
-    T g = T(2) * coef * im;
-    lam[i] = cpx<T>{l.x * cs - l.y * sn + g * p.x, l.y * cs + l.x * sn + g * p.y};
+    double2 p = psi_in[i], l = lam[i];
+    double ph = coef * (p.x * p.x + p.y * p.y - shift);
+    double sn, cs;
+    sincos(ph, &sn, &cs);
+    double2 po{p.x * cs + p.y * sn, p.y * cs - p.x * sn};          // exp(-i ph) p
+    double im = l.x * po.y - l.y * po.x;                                 // Im(conj(l) po)
+    double g = 2.0 * coef * im;
+    lam[i] = double2{l.x * cs - l.y * sn + g * p.x, l.y * cs + l.x * sn + g * p.y};
   }
 }
 
@@ -49,19 +47,14 @@ __global__ void k_phase_grad(const cpx<T>* __restrict__ psi, const cpx<T>* __res
   }
 }
 
-template <typename T> cudaError_t launch_nonlinear(cpx<T>* psi, long long npts, double coef, double shift, cudaStream_t s) {
-  k_nonlinear<T><<<grid_for(npts, 256), 256, 0, s>>>(psi, npts, (T)coef, (T)shift);
+cudaError_t launch_nonlinear(double2* psi, long long npts, double coef, double shift, cudaStream_t s) {
+  k_nonlinear<<<grid_for(npts, 256), 256, 0, s>>>(psi, npts, coef, shift);
   return cudaGetLastError();
 }
-template <typename T>
-cudaError_t launch_vjp_nonlinear(const cpx<T>* psi_in, cpx<T>* lam, long long npts, double coef, double shift, cudaStream_t s) {
-  k_vjp_nonlinear<T><<<grid_for(npts, 256), 256, 0, s>>>(psi_in, lam, npts, (T)coef, (T)shift);
+cudaError_t launch_vjp_nonlinear(const double2* psi_in, double2* lam, long long npts, double coef, double shift, cudaStream_t s) {
+  k_vjp_nonlinear<<<grid_for(npts, 256), 256, 0, s>>>(psi_in, lam, npts, coef, shift);
   return cudaGetLastError();
 }
-template cudaError_t launch_nonlinear<float>(cpx<float>*, long long, double, double, cudaStream_t);
-template cudaError_t launch_nonlinear<double>(cpx<double>*, long long, double, double, cudaStream_t);
-template cudaError_t launch_vjp_nonlinear<float>(const cpx<float>*, cpx<float>*, long long, double, double, cudaStream_t);
-template cudaError_t launch_vjp_nonlinear<double>(const cpx<double>*, cpx<double>*, long long, double, double, cudaStream_t);
 
 }  // namespace gp
 

@@ -484,6 +484,24 @@ gp_status step_all(gp_plan* p, void* const* psi, int nsteps) {
   return run_items(p, groups, epi, psi, s);
 }
 
+gp_status kinetic_block(gp_plan* p, int field, void* psi, double sk) {
+  FieldPlan& F = p->f[field];
+  Group G;
+  G.fields.push_back(field);
+  G.n = F.n;
+  G.fp64 = F.fp64;
+  std::vector<void*> ptrs(p->f.size(), nullptr);
+  ptrs[field] = psi;
+  const bool pl = !G.fp64 && plane_on(p, G.n);
+  if (pl) {
+    gp_status st = ensure_plane_sync(p, plane_sync_ints(G.n, 1));
+    if (st != GP_OK) return st;
+  }
+  std::vector<Item> items;
+  k_block(items, 0, sk, pl);
+  return run_items(p, {G}, items, ptrs.data(), p->stream);
+}
+
 gp_status step_field(gp_plan* p, int field, void* psi, int nsteps) {
   // a one-field view of the plan (used by the adjoint's recomputation)
   std::vector<void*> ptrs(p->f.size(), nullptr);

@@ -6,10 +6,11 @@
 // explicit at the old level.  The implicit part is diagonal in Fourier space:
 //   F phi' = [ (1 - a) F phi + dtau F(rest) ] / (1 + a),   a = dtau alpha |k|^2 / 2,
 //   rest   = -i v . grad phi - |v|^2 / (4 alpha) phi + beta (1 - |phi|^2) phi.
-// Per step: the field's spectrum F phi is kept from the previous step, so a step is three
-// inverse transforms (grad phi, one launch per axis for the three components), one forward
-// transform (rest) and one inverse (phi'), plus three pointwise kernels.  The velocity is
-// evaluated from the grid coordinates inside the kernels (no velocity arrays).
+// The field's spectrum F phi is kept from the previous step.  float64: a step is three inverse
+// transforms (grad phi), one forward transform (rest) and one inverse (phi'), plus three pointwise
+// kernels.  float32: four sweeps in which each component of grad phi branches off the inverse
+// transform of phi at its own axis (see below).  The velocity is evaluated from the grid
+// coordinates inside the kernels (no velocity arrays).
 // Optional L2 renormalisation (the normalised gradient flow): after each step phi and F phi
 // are rescaled on the device to the mean |phi|^2 the field had on entry (float64 sums).
 // E_v = < 2 alpha^2 |grad phi - i v phi / (2 alpha)|^2 + alpha beta (|phi|^2 - 1)^2 >.
@@ -23,17 +24,12 @@
 //     is an integer combination of grid indices times 2 pi / N and is reduced modulo N exactly.
 #include <cmath>
 
+#include "gp_argle.cuh"
+#include "gp_deriv.cuh"
 #include "gp_internal.h"
 #include "gp_reduce.cuh"
 
 namespace gp {
-
-enum { FLOW_NONE = 0, FLOW_TG = 1, FLOW_ABC = 2 };
-
-struct Flow {
-  int kind;
-  double A, B, C;
-};
 
 // Per-axis tables of the flows' trigonometric factors (x = 2 pi i / N), formed once per call in
 // float64 with sincospi: [sin(2 pi i/N) | cos(2 pi i/N) | sin(4 pi i/N) |
@@ -53,34 +49,6 @@ __global__ void k_flow_tables(double* td, float* tf, int n) {
     td[q * n + i] = v[q];
     tf[q * n + i] = (float)v[q];
   }
-}
-
-// velocity at grid point (ix, iy, iz) from the tables, in the precision S of the tables
-template <typename S>
-__device__ __forceinline__ void flow_tab(const Flow& f, const S* __restrict__ tab, int ix, int iy, int iz, int n, S* v) {
-  v[0] = v[1] = v[2] = S(0);
-  if (f.kind == FLOW_NONE) return;
-  const S* s1 = tab;
-  const S* c1 = tab + n;
-  if (f.kind == FLOW_TG) {
-    const S cz = c1[iz];
-    v[0] = s1[ix] * c1[iy] * cz;
-    v[1] = -c1[ix] * s1[iy] * cz;
-    return;
-  }
-  const S A = (S)f.A, B = (S)f.B, C = (S)f.C;
-  S vx = S(0), vy = S(0), vz = S(0);
-#pragma unroll
-  for (int k = 0; k < 2; ++k) {
-    const S* sk = tab + 2 * k * n;
-    const S* ck = sk + n;
-    vx += B * ck[iy] + C * sk[iz];
-    vy += C * ck[iz] + A * sk[ix];
-    vz += A * ck[ix] + B * sk[iy];
-  }
-  v[0] = vx;
-  v[1] = vy;
-  v[2] = vz;
 }
 
 __device__ __forceinline__ int kwave(int i, int n) { return i < (n + 1) / 2 ? i : i - n; }
@@ -255,16 +223,6 @@ static inline unsigned agrid(long long n) {
   return (unsigned)(b < 1 ? 1 : (b > 152LL * 16 ? 152LL * 16 : b));
 }
 
-template <typename T> static cudaError_t transform(gp_plan* p, FieldPlan& F, cpx<T>** xs, int count, bool inverse,
-                                                   cudaStream_t s) {
-  if constexpr (sizeof(T) == 4) return fft3_many(p, F, xs, count, inverse, s);
-  for (int k = 0; k < count; ++k) {
-    cudaError_t e = fft3<T>(F, xs[k], inverse, s);
-    if (e != cudaSuccess) return e;
-  }
-  return cudaSuccess;
-}
-
 // per-block maxima of |phi - old|^2 (a maximum is exact in any precision)
 template <typename T>
 __global__ void k_maxdiff2(const cpx<T>* __restrict__ phi, const cpx<T>* __restrict__ old, long long npts, double* part) {
@@ -286,6 +244,63 @@ __global__ void k_maxdiff2(const cpx<T>* __restrict__ phi, const cpx<T>* __restr
   }
 }
 
+#define GP_DECL(L) extern template struct ArgleLaunch<L>;
+GP_SIZES(GP_DECL)
+#undef GP_DECL
+template <class F> static cudaError_t argle_len(int n, F&& f) {
+  switch (n) {
+#define GP_CASE(L) case L: return f(ArgleLaunch<L>{});
+    GP_SIZES(GP_CASE)
+#undef GP_CASE
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+// float32: E_v's terms of one axis (gp_deriv.cuh): |d_j phi - i v_j phi / (2 alpha)|^2 and, with the x axis, (|phi|^2 - 1)^2
+template <int AXIS_> struct EnergyEpi : DerivEpi {
+  static constexpr int AXIS = AXIS_;
+  Flow flow;
+  const float* tab;
+  float h;         // 1 / (2 alpha)
+  unsigned n;
+  double* part;    // [block][2]
+  using State = Sums<float, 2>;
+  __device__ __forceinline__ float2 point(State& st, long i, float2 p, float2 g, float) const {
+    const unsigned q = (unsigned)i, iy = q / n;
+    const float w = flow_comp<AXIS>(flow, tab, q - iy * n, iy % n, iy / n, n) * h;
+    const float re = g.x + w * p.y, im = g.y - w * p.x;
+    float rho, r = 0.0f;
+    if constexpr (AXIS == 0) r = rho_minus_one<float>(p, &rho);
+    const float v[2] = {re * re + im * im, r * r};
+    st.add(v);
+    return g;
+  }
+  __device__ __forceinline__ void put(long, float2) const {}
+  __device__ __forceinline__ void finish(State& st) const {
+    st.flush();
+    __shared__ double red[32][2];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    const int lanes = (int)min(32u, blockDim.x);
+    const unsigned mask = lanes == 32 ? 0xffffffffu : (1u << lanes) - 1u;
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      double s = st.d[a];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        const double t = __shfl_down_sync(mask, s, o);
+        if (lane + o < lanes) s += t;
+      }
+      if (lane == 0) red[w][a] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2) {
+      double s = red[0][threadIdx.x];
+      for (int q = 1; q < nw; ++q) s += red[q][threadIdx.x];
+      part[(size_t)blockIdx.x * 2 + threadIdx.x] = s;
+    }
+  }
+};
+
 // Convergence checks of a run (eqn:crit1, eqn:crit2): every `every`-th step and the last one
 // evaluate ||phi^{n+1} - phi^n||_inf / dtau and |E_v(phi^{n+1}) - E_v(phi^n)| / (dtau E_v(phi^n));
 // the run stops after the first checked step with crit1 <= eps (eps <= 0: never).
@@ -306,7 +321,9 @@ static gp_status argle_impl(gp_plan* p, int field, cpx<T>* phi, Flow flow, doubl
   const size_t fb = (size_t)npts * sizeof(cpx<T>);
   const unsigned g = agrid(npts);
   const int nf = chk.every > 0 ? 5 : 4;
-  gp_status st = ensure_ws(p, field, nf * fb + (size_t)(2 * g + 16 + 4 * n) * sizeof(double) + (size_t)4 * n * sizeof(float));
+  constexpr int EV = 3 * DERIV_BLOCKS;           // float32: rows of E_v's per-block sums
+  const size_t np = 2 * (size_t)(sizeof(T) == 4 && EV > (int)g ? EV : g);
+  gp_status st = ensure_ws(p, field, nf * fb + (np + 16 + 4 * n) * sizeof(double) + (size_t)4 * n * sizeof(float));
   if (st != GP_OK) return st;
   cpx<T>* ph = (cpx<T>*)F.ws;
   cpx<T>* w1 = ph + npts;
@@ -316,7 +333,7 @@ static gp_status argle_impl(gp_plan* p, int field, cpx<T>* phi, Flow flow, doubl
   double* part = (double*)(ph + (size_t)nf * npts);
   // red: [0] mass sum, [1] target mean |phi|^2, [2..3] energy sums, [4..5] E_v sums before and
   // [6..7] after a checked step, [8] max |phi^{n+1} - phi^n|^2
-  double* red = part + 2 * g;
+  double* red = part + np;
   double* tab_d = red + 16;                      // flow tables, float64 and float32
   float* tab_f = (float*)(tab_d + 4 * n);
   const T* tab = (const T*)(sizeof(T) == 8 ? (const void*)tab_d : (const void*)tab_f);
@@ -324,16 +341,29 @@ static gp_status argle_impl(gp_plan* p, int field, cpx<T>* phi, Flow flow, doubl
   k_flow_tables<<<(n + 127) / 128, 128, 0, s>>>(tab_d, tab_f, n);
   GP_CUDA(p, cudaGetLastError());
   const double alpha = F.alpha, beta = F.beta, dn = (double)npts;
-  cpx<T>* grads[3] = {w1, w2, w3};
-  // E_v sums of the current phi into dst[0..1] (enqueued only; uses w1..w3)
+  // E_v sums of the current phi into dst[0..1] (enqueued only; float64: uses w1..w3)
   auto energy_sums = [&](double* dst) -> gp_status {
-    GP_CUDA(p, cudaMemcpyAsync(w1, phi, fb, cudaMemcpyDeviceToDevice, s));
-    GP_CUDA(p, transform<T>(p, F, &w1, 1, false, s));
-    k_grad_spec<T><<<g, 256, 0, s>>>(w1, w1, w2, w3, n);   // in place: w1 is read before it is written
-    GP_CUDA(p, cudaGetLastError());
-    GP_CUDA(p, transform<T>(p, F, grads, 3, true, s));
-    k_energy_v<T><<<g, 256, 0, s>>>(phi, w1, w2, w3, n, flow, tab, alpha, part);
-    k_reduce<<<1, 256, 0, s>>>(part, (int)g, 2, dst);
+    if constexpr (sizeof(T) == 4) {
+      GP_CUDA(p, cudaMemsetAsync(part, 0, (size_t)EV * 2 * sizeof(double), s));
+      const DerivArgs da{phi, (const tw_t<float>*)F.t32.tw_fwd, (const tw_t<float>*)F.t32.tw_inv};
+      auto axis = [&](auto e) {
+        e.flow = flow, e.tab = tab, e.h = (float)(1.0 / (2.0 * alpha)), e.n = (unsigned)n;
+        e.part = part + (size_t)decltype(e)::AXIS * DERIV_BLOCKS * 2;
+        return deriv(n, da, e, s);
+      };
+      GP_CUDA(p, axis(EnergyEpi<0>{}));
+      GP_CUDA(p, axis(EnergyEpi<1>{}));
+      GP_CUDA(p, axis(EnergyEpi<2>{}));
+      k_reduce<<<1, 256, 0, s>>>(part, EV, 2, dst);
+    } else {
+      GP_CUDA(p, cudaMemcpyAsync(w1, phi, fb, cudaMemcpyDeviceToDevice, s));
+      GP_CUDA(p, fft3<T>(F, w1, false, s));
+      k_grad_spec<T><<<g, 256, 0, s>>>(w1, w1, w2, w3, n);   // in place: w1 is read before it is written
+      GP_CUDA(p, cudaGetLastError());
+      for (cpx<T>* w : {w1, w2, w3}) GP_CUDA(p, fft3<T>(F, w, true, s));
+      k_energy_v<T><<<g, 256, 0, s>>>(phi, w1, w2, w3, n, flow, tab, alpha, part);
+      k_reduce<<<1, 256, 0, s>>>(part, (int)g, 2, dst);
+    }
     GP_CUDA(p, cudaGetLastError());
     return GP_OK;
   };
@@ -350,23 +380,44 @@ static gp_status argle_impl(gp_plan* p, int field, cpx<T>* phi, Flow flow, doubl
       GP_CUDA(p, cudaGetLastError());
     }
     GP_CUDA(p, cudaMemcpyAsync(ph, phi, fb, cudaMemcpyDeviceToDevice, s));
-    GP_CUDA(p, transform<T>(p, F, &ph, 1, false, s));
+    if constexpr (sizeof(T) == 4) GP_CUDA(p, fft3_many(p, F, &ph, 1, false, s));
+    else GP_CUDA(p, fft3<T>(F, ph, false, s));
+    auto checked = [&](int it) { return chk.every > 0 && ((it + 1) % chk.every == 0 || it + 1 == nsteps); };
+    [[maybe_unused]] const int nv = flow.kind == FLOW_NONE ? 0 : (flow.kind == FLOW_TG ? 2 : 3);
+    [[maybe_unused]] bool mixed = false;           // float32: w1 (and w2) hold the mixed form of phi
     for (int it = 0; it < nsteps; ++it) {
-      const bool check = chk.every > 0 && ((it + 1) % chk.every == 0 || it + 1 == nsteps);
+      const bool check = checked(it);
       if (check) {
         GP_CUDA(p, cudaMemcpyAsync(old, phi, fb, cudaMemcpyDeviceToDevice, s));
         st = energy_sums(red + 4);
         if (st != GP_OK) return st;
       }
-      k_grad_spec<T><<<g, 256, 0, s>>>(ph, w1, w2, w3, n);
-      GP_CUDA(p, cudaGetLastError());
-      GP_CUDA(p, transform<T>(p, F, grads, 3, true, s));
-      k_argle_rest<T><<<g, 256, 0, s>>>(phi, w1, w2, w3, n, flow, tab, alpha, beta);
-      GP_CUDA(p, cudaGetLastError());
-      GP_CUDA(p, transform<T>(p, F, &w1, 1, false, s));
-      k_argle_combine<T><<<g, 256, 0, s>>>(ph, w1, phi, n, dtau, alpha);
-      GP_CUDA(p, cudaGetLastError());
-      GP_CUDA(p, transform<T>(p, F, &phi, 1, true, s));
+      if constexpr (sizeof(T) == 4) {
+        ArgleStep a{w1, w3, w2, ph, w1, (const tw_t<float>*)F.t32.tw_fwd, (const tw_t<float>*)F.t32.tw_inv, tab, flow,
+                    (float)(1.0 / (4.0 * alpha)), (float)beta, (float)(0.5 * dtau * alpha), (float)dtau};
+        if (!mixed) GP_CUDA(p, argle_len(n, [&](auto l) { return l.z(a, false, nv == 3, s); }));
+        if (nv == 0) GP_CUDA(p, fft1_many(p, F, &w1, 1, 1, true, s));
+        else GP_CUDA(p, argle_len(n, [&](auto l) { return l.y(a, nv, s); }));
+        GP_CUDA(p, argle_len(n, [&](auto l) { return l.x(a, nv, s); }));
+        GP_CUDA(p, fft1_many(p, F, &w1, 1, 1, false, s));
+        mixed = !(renorm || check || it + 1 == nsteps || checked(it + 1));
+        if (!mixed) a.dst = phi;
+        GP_CUDA(p, argle_len(n, [&](auto l) { return l.z(a, true, mixed && nv == 3, s); }));
+        if (!mixed) {
+          GP_CUDA(p, fft1_many(p, F, &phi, 1, 1, true, s));
+          GP_CUDA(p, fft1_many(p, F, &phi, 1, 0, true, s));
+        }
+      } else {
+        k_grad_spec<T><<<g, 256, 0, s>>>(ph, w1, w2, w3, n);
+        GP_CUDA(p, cudaGetLastError());
+        for (cpx<T>* w : {w1, w2, w3}) GP_CUDA(p, fft3<T>(F, w, true, s));
+        k_argle_rest<T><<<g, 256, 0, s>>>(phi, w1, w2, w3, n, flow, tab, alpha, beta);
+        GP_CUDA(p, cudaGetLastError());
+        GP_CUDA(p, fft3<T>(F, w1, false, s));
+        k_argle_combine<T><<<g, 256, 0, s>>>(ph, w1, phi, n, dtau, alpha);
+        GP_CUDA(p, cudaGetLastError());
+        GP_CUDA(p, fft3<T>(F, phi, true, s));
+      }
       if (renorm) {
         k_mass<T><<<g, 256, 0, s>>>(phi, npts, part);
         k_reduce<<<1, 256, 0, s>>>(part, (int)g, 1, red);

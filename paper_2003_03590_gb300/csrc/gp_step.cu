@@ -44,12 +44,11 @@ int sweep_variant(gp_plan* p, int n, int axis, int op) {
 //   y and z up to 128 points: one step of 24 fields of 64^3 75 us with TMA kernels, 69 without, of 16 fields
 //     of 96^3 251 / 242, of 8 fields of 128^3 220 / 203 (a CTA has few tiles to pipeline); at 192 two
 //     stages: z inverse-N-forward 45.6 / 37.8 / 37.3 (three stages / one tile per CTA / two stages);
-//   z at 1024 with one transform: 6840 / 5000 (128-byte rows without the stages for them).
+//   z at 1024, TMA / one tile per CTA: forward 3470 / 4900, inverse-N-forward 5440 / 7790.
 static int default_variant(int n, int axis, int op) {
   if (op == OP_PLANE) return n == 256 ? VARIANT_TMA : VARIANT_PLAIN;
   if (axis == 0 || n <= 128) return VARIANT_PLAIN;
   if (n == 192) return VARIANT_TMA_2STAGE;
-  if (n == 1024 && axis == 2 && op != OP_INV_N_FWD) return VARIANT_PLAIN;
   return VARIANT_TMA;
 }
 int kernel_variant(gp_plan* p, int n, int axis, int op) {

@@ -37,7 +37,7 @@ template <int L> static void box_of(int axis, cuuint32_t box[3]) {
   } else if (axis == 1) {
     box[0] = TmaStrided<L>::B; box[1] = TmaStrided<L>::BOX; box[2] = 1;
   } else {
-    box[0] = warp_z_pencils<L>(); box[1] = 1; box[2] = TmaStrided<L>::BOX;
+    box[0] = warp_ok<L>() ? WARP_Z_PENCILS : TmaStrided<L>::B; box[1] = 1; box[2] = TmaStrided<L>::BOX;
   }
 }
 

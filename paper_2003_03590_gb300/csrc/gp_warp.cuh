@@ -24,6 +24,7 @@
 #include <type_traits>
 
 #include "gp_tma.cuh"
+#include "gp_ztile.cuh"
 
 namespace gp {
 
@@ -35,11 +36,11 @@ template <int L> __host__ __device__ constexpr bool warp_ok() { return L >= 256;
 // its y sweeps: not at 512, where the block kernel of gp_tma.cuh streams at 94% of the copy rate
 // (336 us against 364)
 template <int L> __host__ __device__ constexpr bool warp_axis(int axis) { return warp_ok<L>() && !(L == 512 && axis == 1); }
-// pencils of a z tile: at 512 16 (128-byte rows).  A z-pencil's elements lie one z-plane apart and a
+// pencils of a z tile: from 256 points on 16 (128-byte rows).  A z-pencil's elements lie one z-plane apart and a
 // copy of z tiles runs at a fixed number of rows per second (512^3: 64-byte rows 675 us, 128-byte
-// rows 361 us, 256-byte rows 338 us; 1024^3: 7157, 3581, 2786 us); at 1024 a stage of 16 pencils
-// would be 128 KB.
-template <int L> __host__ __device__ constexpr int warp_z_pencils() { return L == 1024 ? 8 : 16; }
+// rows 361 us, 256-byte rows 338 us; 1024^3: 7157, 3581, 2786 us); at 1024 a stage of 16 pencils is
+// 128 KB and the z sweeps have a kernel of their own (gp_ztile.cuh).
+constexpr int WARP_Z_PENCILS = 16;
 
 __device__ __forceinline__ float2 lds2(uint32_t a) {
   float2 v;
@@ -352,7 +353,7 @@ template <int L> __host__ __device__ constexpr WarpCfg warp_cfg(int axis, int v)
     return v == 2 ? WarpCfg{8, 3, 2, 2} : WarpCfg{8, 6, 4, 1};   // x
   }
   if (axis == 0) return v == 2 ? WarpCfg{4, 3, 2, 2} : WarpCfg{4, 6, 4, 1};
-  return v == 1 ? WarpCfg{8, 2, 1, 1} : (v == 2 ? WarpCfg{8, 3, 2, 1} : WarpCfg{8, 3, 1, 1});
+  return v == 1 ? WarpCfg{8, 2, 1, 1} : (v == 2 ? WarpCfg{8, 3, 2, 1} : WarpCfg{8, 3, 1, 1});   // y
 }
 
 template <int L> struct WarpLaunch {
@@ -386,9 +387,10 @@ template <int L> struct WarpLaunch {
       Occ q{};
       fill<0, 0>(q);
       if constexpr (warp_axis<L>(1)) fill<1, 0>(q), fill<1, 1>(q);
-      fill<2, 0>(q), fill<2, 1>(q);
+      if constexpr (!ztile_ok<L>()) fill<2, 0>(q), fill<2, 1>(q);
       if constexpr (NV > 2 && warp_axis<L>(1)) fill<1, 2>(q);
-      if constexpr (NV > 2) fill<0, 2>(q), fill<2, 2>(q);
+      if constexpr (NV > 2) fill<0, 2>(q);
+      if constexpr (NV > 2 && !ztile_ok<L>()) fill<2, 2>(q);
       return q;
     }();
     return o;
@@ -414,20 +416,27 @@ template <int L> struct WarpLaunch {
 #undef GP_R
   }
   static cudaError_t launch(const TmaSweepArgs& a, int cap, int stages, int groups, cudaStream_t s) {
+    if constexpr (ztile_ok<L>()) {
+      if (a.axis == 2 && (groups == 1 || groups == 2)) return ZTileLaunch<L>::launch(a, s);   // whatever the variant
+    }
     if constexpr (!warp_axis<L>(1)) {
       if (a.axis == 1 && groups == 1) return TmaLaunch<L>::launch(a, cap, stages, 1, s);
     }
     if (groups == 2) {
       if constexpr (NV > 2) {
         if (a.axis == 0) return run_op<0, 2>(a, cap, s);
-        if (a.axis == 2) return run_op<2, 2>(a, cap, s);
+        if constexpr (!ztile_ok<L>()) {
+          if (a.axis == 2) return run_op<2, 2>(a, cap, s);
+        }
         if constexpr (warp_axis<L>(1)) return run_op<1, 2>(a, cap, s);
         else return TmaLaunch<L>::launch(a, cap, 3, 1, s);
       }
     }
     if (groups != 1) return cudaErrorInvalidValue;
     if (a.axis == 0) return run_op<0, 0>(a, cap, s);
-    if (a.axis == 2) return stages == 2 ? run_op<2, 1>(a, cap, s) : run_op<2, 0>(a, cap, s);
+    if constexpr (!ztile_ok<L>()) {
+      if (a.axis == 2) return stages == 2 ? run_op<2, 1>(a, cap, s) : run_op<2, 0>(a, cap, s);
+    }
     if constexpr (warp_axis<L>(1)) return stages == 2 ? run_op<1, 1>(a, cap, s) : run_op<1, 0>(a, cap, s);
     else return cudaErrorInvalidValue;
   }

@@ -370,7 +370,7 @@ __device__ __forceinline__ void pass_compute(cpx<T>* v, int t, const tw_t<T>* __
       const int jm = j % NS;
 #pragma unroll
       for (int r = 1; r < R; ++r) {
-        const tw_t<T>* q = tw + OFF + jm * (R - 1) + (r - 1);
+        const tw_t<T>* q = tw + OFF + (r - 1) * NS + jm;
         if constexpr (TW_SH) v[b * R + r] = twmul(v[b * R + r], *q);
         else v[b * R + r] = twmul(v[b * R + r], __ldg(q));
       }

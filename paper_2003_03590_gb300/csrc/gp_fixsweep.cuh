@@ -136,9 +136,9 @@ template <int L, bool INV, int I> __device__ __forceinline__ void fix_pass(cfix*
 #pragma unroll
   for (int b = 0; b < E / R; ++b) {
     if constexpr (NS > 1) {
-      const ufix2* q = tw + tw_offset<L, INV>(I) + ((t + b * TP) % NS) * (R - 1);
+      const ufix2* q = tw + tw_offset<L, INV>(I) + (t + b * TP) % NS;
 #pragma unroll
-      for (int r = 1; r < R; ++r) v[b * R + r] = ftwmul(v[b * R + r], ldg_u2(q + r - 1));
+      for (int r = 1; r < R; ++r) v[b * R + r] = ftwmul(v[b * R + r], ldg_u2(q + (r - 1) * NS));
     }
     fdft<R, INV>(v + b * R);
   }

@@ -530,25 +530,18 @@ struct NoAllocDevice {
 };
 static NoAllocDevice g_na_dev[64];
 
-// Stockham twiddles (same definition as the plan's tables) written into a fixed host array.
+// a length's twiddles, as the plan's tables hold them, into a fixed host array
 static int noalloc_twiddles(int n, bool inv, float4* out, int cap) {
-  const int np = plan_np(n);
-  int ns = 1, k = 0;
-  for (int i = 0; i < np; ++i) {
-    const int R = plan_radix_fwd(n, inv ? np - 1 - i : i);
-    for (int jm = 0; jm < ns; ++jm)
-      for (int r = 1; r < R; ++r) {
-        if (k >= cap) return -1;
-        const long long den = (long long)ns * R, num = ((long long)r * jm) % den;
-        const double ang = (inv ? 2.0 : -2.0) * M_PI * (double)num / (double)den;
-        float ch, cl, sh, sl;
-        split_hilo(std::cos(ang), &ch, &cl);
-        split_hilo(std::sin(ang), &sh, &sl);
-        out[k++] = make_float4(ch, sh, cl, sl);
-      }
-    ns *= R;
+  std::vector<double> re, im;
+  twiddles(n, inv, re, im);
+  if ((int)re.size() > cap) return -1;
+  for (size_t k = 0; k < re.size(); ++k) {
+    float ch, cl, sh, sl;
+    split_hilo(re[k], &ch, &cl);
+    split_hilo(im[k], &sh, &sl);
+    out[k] = make_float4(ch, sh, cl, sl);
   }
-  return k;
+  return (int)re.size();
 }
 
 // Once per device, with that device current: resolve the device addresses of the arrays

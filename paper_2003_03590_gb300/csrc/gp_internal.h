@@ -47,6 +47,7 @@ cudaError_t ensemble_run(gp_plan* p, const std::vector<int>& fields, void* const
                          cudaStream_t s, int skip = 0);
 
 bool supported_n(int n);
+void twiddles(int n, bool inv, std::vector<double>& re, std::vector<double>& im);   // a direction's table
 void split_hilo(double v, float* hi, float* lo);   // see gp_plan.cu
 int plan_np(int n);           // number of radix passes for length n
 int plan_radix_fwd(int n, int i);

@@ -81,7 +81,7 @@ gp_status cuda_fail(gp_plan* p, cudaError_t e, const char* what) {
 // (r-1) NS + jm holds exp(sign 2 pi i r jm / (NS R)), jm < NS, 1 <= r < R: the lanes of a warp take
 // consecutive jm of the same r, contiguous (with jm (R-1) + (r-1) each lane of an x sweep read a cache
 // line of its own: GB300, 512^3 x sweep with K 527 us, now 505 us, 128^3 imaginary-time step 84 and 82).
-static void twiddles(int n, bool inv, std::vector<double>& re, std::vector<double>& im) {
+void twiddles(int n, bool inv, std::vector<double>& re, std::vector<double>& im) {
   const int np = plan_np(n);
   re.clear();
   im.clear();

@@ -352,7 +352,7 @@ template <int L, bool INV> __host__ __device__ constexpr int tw_offset(int i) {
 template <int L, bool INV> __host__ __device__ constexpr int tw_size() { return tw_offset<L, INV>(Plan<L>::NP); }
 
 // ---------------------------------------------------------------- pencil engine
-// Layout functor Lay: int smem_index(int pencil, int pos).  Registers v[E]:
+// Layout Lay: at<INV, X>(pencil, pos), the element's index in exchange X (between passes X and X + 1).  Registers v[E]:
 // at the input of pass i (radix R) v[b R + r] holds x[t + b TP + r L/R].
 // TW_SH: the twiddle table has been copied to shared memory (plain loads), else read through
 // the read-only data cache.
@@ -392,7 +392,7 @@ __device__ __forceinline__ void pass_store(const cpx<T>* v, int t, int p, cpx<T>
     const int j = t + b * TP;
     const int idxD = (j / NS) * NS * R + (j % NS);
 #pragma unroll
-    for (int r = 0; r < R; ++r) sm[lay(p, idxD + r * NS)] = v[b * R + r];
+    for (int r = 0; r < R; ++r) sm[lay.template at<INV, I>(p, idxD + r * NS)] = v[b * R + r];
   }
 }
 
@@ -406,7 +406,7 @@ __device__ __forceinline__ void pass_load(cpx<T>* v, int t, int p, const cpx<T>*
   for (int b = 0; b < E / R; ++b) {
     const int j = t + b * TP;
 #pragma unroll
-    for (int r = 0; r < R; ++r) v[b * R + r] = sm[lay(p, j + r * (L / R))];
+    for (int r = 0; r < R; ++r) v[b * R + r] = sm[lay.template at<INV, I - 1>(p, j + r * (L / R))];
   }
 }
 

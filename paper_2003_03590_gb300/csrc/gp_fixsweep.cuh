@@ -150,7 +150,7 @@ template <int L, bool INV, int I, class Lay> __device__ __forceinline__ void fix
     const int j = t + b * TP, d = (j / NS) * NS * R + (j % NS);
 #pragma unroll
     for (int r = 0; r < R; ++r)
-      *reinterpret_cast<longlong2*>(sm + lay(p, d + r * NS)) = make_longlong2(v[b * R + r].x, v[b * R + r].y);
+      *reinterpret_cast<longlong2*>(sm + lay.template at<INV, I>(p, d + r * NS)) = make_longlong2(v[b * R + r].x, v[b * R + r].y);
   }
 }
 template <int L, bool INV, int I, class Lay> __device__ __forceinline__ void fix_load(cfix* v, int t, int p, const cfix* sm, const Lay& lay) {
@@ -159,7 +159,7 @@ template <int L, bool INV, int I, class Lay> __device__ __forceinline__ void fix
   for (int b = 0; b < E / R; ++b)
 #pragma unroll
     for (int r = 0; r < R; ++r) {
-      const longlong2 q = *reinterpret_cast<const longlong2*>(sm + lay(p, t + b * TP + r * (L / R)));
+      const longlong2 q = *reinterpret_cast<const longlong2*>(sm + lay.template at<INV, I - 1>(p, t + b * TP + r * (L / R)));
       v[b * R + r] = cfix{q.x, q.y};
     }
 }

@@ -36,11 +36,11 @@ int sweep_variant(gp_plan* p, int n, int axis, int op) {
 
 // The kernel of a sweep kind when none was chosen for the plan, by the length.  Measured on GB300, us per
 // launch of one field (the batched steps order the same way):
-//   y, x, y as the fused plane kernel / as three sweeps: 32^3 27 / 13, 64^3 30 / 15, 96^3 39 / 26, 128^3
-//     39 / 31, 192^3 113 / 92, 256^3 144 / 156, 512^3 1655 / 1260, 1024^3 12800 / 10300: fused where its
+//   y, x, y as the fused plane kernel / as three sweeps: 32^3 27 / 15, 64^3 29 / 15, 96^3 37 / 23, 128^3
+//     39 / 30, 192^3 103 / 82, 256^3 144 / 153, 512^3 1600 / 1160, 1024^3 11500 / 9240: fused where its
 //     planes both fill the GPU and are few enough to stay in L2, which is 256;
-//   x sweeps (forward, K, inverse), TMA / one tile per CTA: 128^3 16.9 / 14.8, 192^3 55 / 52, 256^3 71 / 66,
-//     512^3 577 / 530, 1024^3 5510 / 5005: rows are contiguous, direct loads lose nothing;
+//   x sweeps (forward, K, inverse), TMA / one tile per CTA: 128^3 16.9 / 14.5, 192^3 45.6 / 41.5, 256^3 71 / 64,
+//     512^3 526 / 491, 1024^3 4440 / 4100: rows are contiguous, direct loads lose nothing;
 //   y and z up to 128 points: one step of 24 fields of 64^3 75 us with TMA kernels, 69 without, of 16 fields
 //     of 96^3 251 / 242, of 8 fields of 128^3 220 / 203 (a CTA has few tiles to pipeline); at 192 two
 //     stages: z inverse-N-forward 45.6 / 37.8 / 37.3 (three stages / one tile per CTA / two stages);

@@ -54,7 +54,23 @@ template <typename T, int L> __host__ __device__ constexpr int contig_batch() {
   while ((L * L) % b) b /= 2;
   return b;
 }
-template <int L> __host__ __device__ constexpr int contig_pitch() { return L + (L >= 16 ? L / 16 : 1); }
+// The x rows' exchange number X (between passes X and X + 1) of direction INV keeps position pos at pos + pos / pad
+// (pad 0: at pos), rows contig_pitch apart: a half-warp's 16 eight-byte accesses (a quarter-warp's 8 of 16 bytes)
+// then fall on different banks, but for 3 to 10% at 32, 48, 96 and 192 points.  The first pass of radix R writes with a
+// stride of R, conflict-free when R is odd; the second one of the inverse transforms of three passes writes blocks of 3
+// consecutive positions.  (With one pad element every 16 in every exchange 192 took 2.0 times the accesses of a
+// conflict-free exchange, 96 and 48 2.0, 32 1.75, 64 and 1024 1.5, 512 and 128 1.25; shared memory and L1 are
+// what bounds x sweeps: GB300, forward-K-inverse, us before -> now: 192^3 49.6 -> 41.5,
+// 512^3 505 -> 491, 1024^3 4600 -> 4100.)
+template <int L, bool INV, int X> __host__ __device__ constexpr int contig_pad() {
+  constexpr int R = radix_of<L, INV>(0);
+  if (L < 32) return 0;   // a thread holds a whole row
+  if (X == 1) return INV ? radix_of<L, false>(0) : 0;
+  return R % 2 ? 0 : (R < 8 && Plan<L>::NP == 2 ? 8 : R);
+}
+template <int L> __host__ __device__ constexpr int contig_pitch() {
+  return L < 32 ? L + 1 : L == 48 ? L + L / 4 : L < 128 || L == 192 ? L + L / 8 : L == 128 ? L + L / 8 + 8 : L + L / 16;
+}
 // CTAs per SM the registers of the capped one-tile-per-CTA kernels must allow (y/z: 256 threads,
 // two per SM, or at 1024 512 threads, one; x: 128 threads, four per SM).  Without a cap the compiler keeps all of a thread's 32
 // loads in flight at once and uses so many registers (~175) that one 8-warp CTA fills the SM
@@ -67,11 +83,14 @@ template <typename T, int L> __host__ __device__ constexpr int rcap_blocks(bool 
 
 struct LayStrided {  // [pos][pencil]
   int B;
-  __device__ __forceinline__ int operator()(int p, int pos) const { return pos * B + p; }
+  template <bool INV, int X> __device__ __forceinline__ int at(int p, int pos) const { return pos * B + p; }
 };
-template <int L> struct LayContig {  // [pencil][pos] with one pad element every 16
-  __device__ __forceinline__ int operator()(int p, int pos) const {
-    return p * contig_pitch<L>() + pos + (L >= 16 ? (pos >> 4) : 0);
+template <int L> struct LayContig {  // [pencil][pos], padded
+  template <bool INV, int X> __device__ __forceinline__ int at(int p, int pos) const {
+    constexpr unsigned D = contig_pad<L, INV, X>();
+    static_assert(L - 1 + (D ? (L - 1) / (D ? D : 1) : 0) < contig_pitch<L>(), "the last position lies in its row");
+    if constexpr (D == 0) return p * contig_pitch<L>() + pos;
+    else return p * contig_pitch<L>() + pos + (int)((unsigned)pos / D);
   }
 };
 

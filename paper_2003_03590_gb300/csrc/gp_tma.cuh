@@ -137,6 +137,7 @@ template <int L> struct TmaContig {
   static constexpr int NT = B * TP;
   static constexpr int TILE = B * L;
   static constexpr int STAGE = B * contig_pitch<L>();     // elements, >= TILE
+  static_assert(STAGE % 16 == 0, "stages of whole 128-byte lines");
   static constexpr int BOX = L > 256 ? 256 : L;
   static constexpr int NBOX = L / BOX;
   static constexpr int S = 3;

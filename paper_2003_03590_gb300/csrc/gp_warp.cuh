@@ -19,7 +19,7 @@
 // XOR on a per-thread base plus an immediate.
 //
 // x tiles (B rows).  The rows are copied one by one (bulk copies) to a pitch of pitch() elements; a
-// row's exchange uses the padded layout pos + pos / 16 inside its own row.
+// row's exchange uses the padded layout pos + pos / R0 inside its own row.
 #pragma once
 #include <type_traits>
 
@@ -109,12 +109,12 @@ template <int L> struct WarpContig {
     nat = row + 8 * t;
   }
   __device__ __forceinline__ uint32_t natural(int c) const { return nat + 8 * c; }
-  // element pos + pos / 16 for pos = R0 (t + b TP) + k (write) and pos = R0 r + t + b TP (read)
+  // element pos + pos / R0 for pos = R0 (t + b TP) + k (write) and pos = R0 r + t + b TP (read, t + b TP < R0)
   template <int R0> __device__ __forceinline__ uint32_t ex_write(int b, int k) const {
-    return row + 8u * (uint32_t)(t * (R0 + R0 / 16)) + 8u * (b * TP * (R0 + R0 / 16) + k + k / 16);
+    return row + 8u * (uint32_t)((R0 + 1) * t) + 8u * (b * TP * (R0 + 1) + k);
   }
   template <int R0> __device__ __forceinline__ uint32_t ex_read(int b, int r) const {
-    return nat + 8u * (R0 * r + b * TP + (R0 * r + b * TP) / 16) + (TP > 16 ? 8u * (uint32_t)(t / 16) : 0u);
+    return nat + 8u * ((R0 + 1) * r + b * TP);
   }
 };
 

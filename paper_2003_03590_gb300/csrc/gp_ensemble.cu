@@ -68,10 +68,11 @@ template <int L> __host__ __device__ constexpr int ens_sub() {
 template <int L> __host__ __device__ constexpr int ens_items_strided() {
   return (L / strided_batch<float, L>()) * L / ens_sub<L>();
 }
-template <int L> __host__ __device__ constexpr int ens_items_contig() { return L * L / contig_batch<float, L>(); }
+template <int L> __host__ __device__ constexpr int ens_rows() { return ENS_THREADS / (L / Plan<L>::E); }   // of an x tile
+template <int L> __host__ __device__ constexpr int ens_items_contig() { return L * L / ens_rows<L>(); }
 template <int L> __host__ __device__ constexpr size_t ens_smem() {
   const size_t s = sizeof(float2) * (size_t)L * strided_batch<float, L>() * ens_sub<L>();
-  const size_t c = sizeof(float2) * (size_t)contig_pitch<L>() * contig_batch<float, L>();
+  const size_t c = sizeof(float2) * (size_t)contig_pitch<L>() * ens_rows<L>();
   return s > c ? s : c;
 }
 
@@ -87,10 +88,10 @@ template <int L> __device__ __noinline__ void ens_stage_item(const EnsField& F, 
   a.ek2 = F.ek2;
   a.nl_shift = F.nl_shift;
   a.scale_inv = 0;
-  static_assert(contig_batch<float, L>() * (L / Plan<L>::E) == ENS_THREADS, "one x tile per CTA");
+  static_assert(ens_rows<L>() * (L / Plan<L>::E) == ENS_THREADS && L * L % ens_rows<L>() == 0, "one x tile per CTA");
   if (kind == 2) {   // x rows: forward x, K(dt) with 1/n^3, inverse x
     a.axis = 0;
-    contig_tile<float, L, OP_FWD_K_INV>(a, item, F.psi, threadIdx.x, sm);
+    contig_tile<float, L, OP_FWD_K_INV, ens_rows<L>()>(a, item, F.psi, threadIdx.x, sm);
     return;
   }
   static_assert(ENS_THREADS % (strided_batch<float, L>() * (L / Plan<L>::E)) == 0, "whole tiles per CTA");

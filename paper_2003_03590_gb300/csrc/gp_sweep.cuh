@@ -49,7 +49,7 @@ template <typename T, int L> __host__ __device__ constexpr int strided_batch() {
 // several CTAs per SM (see rcap_blocks); their x-row CTAs have 128 threads, four per SM
 template <typename T, int L> __host__ __device__ constexpr bool rcapped() { return sizeof(T) == 4 && Plan<L>::E >= 32; }
 template <typename T, int L> __host__ __device__ constexpr int contig_batch() {
-  int b = (rcapped<T, L>() ? 128 : 256) / (L / Plan<L>::E);
+  int b = (sizeof(T) == 4 && Plan<L>::E >= 24 ? 128 : 256) / (L / Plan<L>::E);
   b = b > 64 ? 64 : (b < 1 ? 1 : b);
   while ((L * L) % b) b /= 2;
   return b;
@@ -77,9 +77,14 @@ template <int L> __host__ __device__ constexpr int contig_pitch() {
 // (measured at 512^3: z N-forward 752 us uncapped, 452 us capped).  Kernels of shorter lengths keep
 // the compiler's own choice (naming a minimum of one CTA per SM lifts its default limit and made
 // the 256-point kernels twice as slow).
+// The sweeps of 96 and 192 points (24 elements a thread) are held to 16 warps per SM for y and z, 20 for x, with
+// x CTAs of 128 threads: GB300, 16 fields of 96^3, x sweep 90 -> 83 us, z inverse-N-forward 70 -> 64 us (at 20 warps y
+// and z spill).
 template <typename T, int L> __host__ __device__ constexpr int rcap_blocks(bool contig) {
+  if (Plan<L>::E < 32) return contig ? 5 : 512 / (strided_batch<T, L>() * (L / Plan<L>::E));
   return contig ? 4 : (strided_batch<T, L>() * (L / Plan<L>::E) >= 512 ? 1 : 2);
 }
+template <typename T, int L> __host__ __device__ constexpr bool sweep_capped() { return rcapped<T, L>() || (sizeof(T) == 4 && L >= 96 && Plan<L>::E == 24); }
 
 struct LayStrided {  // [pos][pencil]
   int B;
@@ -283,11 +288,10 @@ __global__ void __launch_bounds__(strided_batch<T, L>() * (L / Plan<L>::E), rcap
 }
 
 // x rows: a tile is B consecutive rows (y, z); the exchanges of a row stay within one warp.
-template <typename T, int L, int OP>
+template <typename T, int L, int OP, int B = contig_batch<T, L>()>
 __device__ __forceinline__ void contig_tile(const SweepArgs<T>& a, long tile, cpx<T>* psi, int tid, cpx<T>* sm) {
   using V = cpx<T>;
   constexpr int TP = L / Plan<L>::E;
-  constexpr int B = contig_batch<T, L>();
   const int p = tid / TP, t = tid % TP;
   const long row = tile * B + p;
   V* base = psi + row * L;
@@ -317,7 +321,7 @@ template <typename T, int L> struct SweepLaunch {
   static constexpr int TP = L / Plan<L>::E;
   static constexpr int BS = strided_batch<T, L>();
   static constexpr int BC = contig_batch<T, L>();
-  static constexpr bool RC = rcapped<T, L>();
+  static constexpr bool RC = sweep_capped<T, L>();
   static size_t smem_strided() { return sizeof(cpx<T>) * (size_t)L * BS; }
   static size_t smem_contig() { return sizeof(cpx<T>) * (size_t)contig_pitch<L>() * BC; }
   // the shared-memory limit of every operation's kernel, set together on the first launch of

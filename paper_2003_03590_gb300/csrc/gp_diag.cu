@@ -263,7 +263,8 @@ static gp_diag diag_finish(const double* acc, const double* hs, int nb, long lon
 // What one axis' derivative kernel does with d_j psi: W_j = u_j + i q_j, transformed forward along
 // this axis already; the sums of |u|^2 / 2, 2 alpha^2 |q|^2 and, over the axis' spectrum, |k_j|^2 |F_j psi|^2
 // and k~_j |F_j psi|^2 (by Parseval over the other two axes these are the sums over the whole spectrum
-// divided by N^2); u_j^2 added up over the axes in uu.  FIRST: also rho - 1, transformed along this axis,
+// divided by N^2); u_j^2 added up over the axes in uu (the field of the LAST axis' result: a row's values are read
+// before its results are written).  FIRST: also rho - 1, transformed along this axis,
 // and its sums.  LAST: the maximum of |u|^2.
 // Per-block results, DIAG_COLS doubles: [0] rho [1] (rho-1)^2 [2] |k|^2 [3 + j] k~_j [6] u^2/2 [7] q
 // [8] max |u|^2; each kernel adds to its blocks' row.
@@ -273,7 +274,7 @@ template <int AXIS_, bool FIRST, bool LAST> struct DiagEpi : DerivEpi {
   static constexpr bool MODES = true, PRE = !FIRST;
   float2* w;            // W of this axis
   float2* w0;           // FIRST: rho - 1
-  float* uu;
+  float2* uu;           // .x
   float alpha2, qa;     // 2 alpha, 2 alpha^2
   double* part;
   int* flag;
@@ -289,7 +290,7 @@ template <int AXIS_, bool FIRST, bool LAST> struct DiagEpi : DerivEpi {
     st.m[0] += (float)(k * k) * a2;
     st.m[1] += (float)kd * a2;
   }
-  __device__ __forceinline__ float pre(long i) const { return uu[i]; }
+  __device__ __forceinline__ float pre(long i) const { return uu[i].x; }
   __device__ __forceinline__ float2 point(State& st, long i, float2 p, float2 g, float before) const {
     float rho;
     const float dm = rho_minus_one<float>(p, &rho);
@@ -301,7 +302,7 @@ template <int AXIS_, bool FIRST, bool LAST> struct DiagEpi : DerivEpi {
     st.m[0] = st.m[1] = 0.0f;
     const float sum = FIRST ? u * u : fmaf(u, u, before);
     if constexpr (LAST) st.umax = fmaxf(st.umax, sum);
-    else uu[i] = sum;
+    else uu[i] = float2{sum, 0.0f};   // whole sectors
     if constexpr (FIRST) {
       st.bad |= !isfinite(dm);
       const float d[2] = {rho, dm * dm};
@@ -359,7 +360,7 @@ template <int AXIS_, bool FIRST, bool LAST> struct DiagEpi : DerivEpi {
 };
 
 template <int AXIS, bool FIRST, bool LAST>
-static cudaError_t diag_axis(FieldPlan& F, const float2* psi, float2* w, float2* w0, float* uu, double* part, int* flag, cudaStream_t s) {
+static cudaError_t diag_axis(FieldPlan& F, const float2* psi, float2* w, float2* w0, float2* uu, double* part, int* flag, cudaStream_t s) {
   DiagEpi<AXIS, FIRST, LAST> e;
   e.w = w;
   e.w0 = w0;
@@ -370,10 +371,10 @@ static cudaError_t diag_axis(FieldPlan& F, const float2* psi, float2* w, float2*
   e.flag = flag;
   return deriv(F.n, DerivArgs{psi, (const tw_t<float>*)F.t32.tw_fwd, (const tw_t<float>*)F.t32.tw_inv}, e, s);
 }
-// psi -> the spectra of rho - 1, W_x, W_y, W_z in w[0..3] and the sums; part: DERIV_BLOCKS rows, zeroed
-// here; uu: one float per point
-static cudaError_t diag_fields(gp_plan* p, FieldPlan& F, const float2* psi, float2* const* w, float* uu, double* part, int* flag,
+// psi -> the spectra of rho - 1, W_x, W_y, W_z in w[0..3] and the sums; part: DERIV_BLOCKS rows, zeroed here
+static cudaError_t diag_fields(gp_plan* p, FieldPlan& F, const float2* psi, float2* const* w, double* part, int* flag,
                                cudaStream_t s) {
+  float2* uu = w[1];
   cudaError_t e = cudaMemsetAsync(part, 0, (size_t)DERIV_BLOCKS * DIAG_COLS * sizeof(double), s);
   if (e == cudaSuccess) e = diag_axis<2, true, false>(F, psi, w[3], w[0], uu, part, flag, s);
   if (e == cudaSuccess) e = diag_axis<1, false, false>(F, psi, w[2], nullptr, uu, part, flag, s);
@@ -398,8 +399,7 @@ static gp_status diag_impl(gp_plan* p, int field, const cpx<T>* psi, gp_diag* ou
   const size_t fb = (size_t)npts * sizeof(cpx<T>);
   const unsigned g = rgrid(npts);
   const size_t rows = sizeof(T) == 4 && g < (unsigned)DERIV_BLOCKS ? (unsigned)DERIV_BLOCKS : g;
-  const size_t ub = sizeof(T) == 4 ? (size_t)npts * sizeof(float) : 0;   // float32: |u|^2 summed axis by axis
-  gp_status st = ensure_ws(p, field, 4 * fb + (size_t)4 * nbins * sizeof(double) + 9 * rows * sizeof(double) + ub);
+  gp_status st = ensure_ws(p, field, 4 * fb + (size_t)4 * nbins * sizeof(double) + 9 * rows * sizeof(double));
   if (st != GP_OK) return st;
   cpx<T>* w0 = (cpx<T>*)F.ws;
   cpx<T>* w1 = w0 + npts;
@@ -419,7 +419,7 @@ static gp_status diag_impl(gp_plan* p, int field, const cpx<T>* psi, gp_diag* ou
     return cudaSuccess;
   };
   if constexpr (sizeof(T) == 4) {
-    GP_CUDA(p, diag_fields(p, F, psi, all, (float*)(part + 9 * rows), part, p->flag, s));
+    GP_CUDA(p, diag_fields(p, F, psi, all, part, p->flag, s));
     k_reduce_cols<<<DIAG_COLS, 256, 0, s>>>(part, DERIV_BLOCKS, DIAG_COLS, DIAG_COLS - 1, p->acc);
     GP_CUDA(p, cudaGetLastError());
   } else {

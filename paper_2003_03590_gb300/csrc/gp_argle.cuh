@@ -10,7 +10,7 @@
 // from its axis on: 6, 9 or 12 one-dimensional transforms a step, where the components' own
 // three-dimensional inverse transforms took 15, plus three pointwise passes.  Where phi itself is
 // wanted (the last step, a renormalisation, a convergence check) the last z sweep writes it to phi,
-// whose y and x transforms follow.  GB300, 128^3, 20 TG steps and the energy: 3.30 ms so before, now 1.68 ms;
+// whose y and x transforms follow.  GB300, 128^3, 20 TG steps and the energy: 3.30 ms so before, now 1.61 ms;
 // ABC 3.42 and 2.04, no flow at 96^3 2.61 and 0.83.  Bound by latency at 16 warps per SM (the fields stay in L2).
 #pragma once
 #include "gp_reduce.cuh"

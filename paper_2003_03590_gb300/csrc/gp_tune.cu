@@ -7,6 +7,8 @@
 //   2  the non-persistent kernel (one tile per CTA, loads and stores by the threads)
 //   3  (y and z) the TMA kernel with two shared-memory stages instead of three: one tile of
 //      look-ahead, one more CTA per SM
+//   4  (lengths from 512 on) the TMA kernel with another split into stages and compute groups
+// (at 1024 every TMA variant of z is the one kernel of gp_ztile.cuh)
 // and keeps the fastest; the fused plane kernel (op 7) is timed against the three sweeps it
 // replaces.  Choices are cached in a small JSON file keyed by the GPU's name.
 #include <cstdio>

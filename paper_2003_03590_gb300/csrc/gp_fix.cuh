@@ -35,6 +35,14 @@ struct ufix2 {   // a table factor c + i s as ((c + 1) / 2, (s + 1) / 2) in unit
   unsigned long long c, s;
 };
 
+// a component v of a table factor as ufix2 holds it.  The product of two rounded unit factors can lie an
+// ulp outside [-1, 1]: it counts as 1 or -1 (unclamped, the sum below would wrap to the other sign).
+inline unsigned long long fix_factor(double v) {
+  if (v >= 1.0) return ~1ull;
+  if (v <= -1.0) return 0;
+  return ((unsigned long long)(long long)std::nearbyint(std::ldexp(v, 62)) << 1) + (1ull << 63);   // (v + 1) 2^63
+}
+
 #define GP_HD __host__ __device__ __forceinline__
 
 // (a b) / 2^64 rounded, the low x low partial product replaced by its mean

@@ -129,16 +129,8 @@ template <> float4 pack<float4>(double c, double s) {
   split_hilo(s, &sh, &sl);
   return make_float4(ch, sh, cl, sl);
 }
-// float64: fixed point, (c + 1) / 2 and (s + 1) / 2 in units of 2^-64, even
-template <> ufix2 pack<ufix2>(double c, double s) {
-  auto u = [](double v) {
-    const double w = std::ldexp(v, 62);                        // exact; |v| <= 1
-    const long long q = (long long)std::nearbyint(w);
-    const unsigned long long r = ((unsigned long long)q << 1) + (1ull << 63);   // (v + 1) 2^63
-    return v >= 1.0 ? ~1ull : r;
-  };
-  return ufix2{u(c), u(s)};
-}
+// float64: fixed point
+template <> ufix2 pack<ufix2>(double c, double s) { return ufix2{fix_factor(c), fix_factor(s)}; }
 
 // cos and sin of 2 pi num / den (0 <= num < den) to about 2^-60: the angle is reduced to the first
 // octant in integers and the Taylor series summed in units of 2^-60

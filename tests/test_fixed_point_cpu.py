@@ -1,0 +1,94 @@
+"""The fixed-point arithmetic of the float64 sweeps (gp_fix.cuh) on the host, against exact integers.
+
+gp_fix.cuh is compiled into a small program by the host compiler; Python's integers are the reference.
+Tolerances: a table component is stored in units of 2^-62 (2^-60 allows four of them); a
+product by a table factor rounds four half products to one unit each: 4 units a component.
+"""
+import os
+import shutil
+import struct
+import subprocess
+from fractions import Fraction
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+SOURCE = r"""
+#include <cstdio>
+#include "gp_fix.cuh"
+// lines "c s x y" (doubles by their bits, integers): the stored factors and (x + i y)(c + i s)
+int main() {
+  unsigned long long bc, bs;
+  long long x, y;
+  while (std::scanf("%llu %llu %lld %lld", &bc, &bs, &x, &y) == 4) {
+    double c, s;
+    std::memcpy(&c, &bc, 8);
+    std::memcpy(&s, &bs, 8);
+    const gp::ufix2 w{gp::fix_factor(c), gp::fix_factor(s)};
+    const gp::cfix z = gp::ftwmul(gp::cfix{x, y}, w);
+    std::printf("%llu %llu %lld %lld\n", w.c, w.s, z.x, z.y);
+  }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def multiply(tmp_path_factory):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc")), "include")
+    if cxx is None or not os.path.exists(os.path.join(cuda, "cuda_runtime.h")):
+        pytest.skip("no host compiler or CUDA headers")
+    d = tmp_path_factory.mktemp("fix")
+    (d / "fix.cpp").write_text(SOURCE)
+    subprocess.run([cxx, "-std=c++17", "-O1", "-I", os.path.join(ROOT, "paper_2003_03590_gb300", "csrc"), "-I", cuda,
+                    str(d / "fix.cpp"), "-o", str(d / "fix")], check=True)
+
+    def run(c, s, x, y):
+        bits = [struct.unpack("<Q", struct.pack("<d", v))[0] for v in np.concatenate([c, s])]
+        m = len(c)
+        text = "".join(f"{bits[i]} {bits[m + i]} {x[i]} {y[i]}\n" for i in range(m))
+        out = subprocess.run([str(d / "fix")], input=text, capture_output=True, text=True, check=True).stdout.split()
+        return [tuple(int(v) for v in out[4 * i:4 * i + 4]) for i in range(m)]
+    return run
+
+
+def pair_table(n, alpha, s):
+    """E[k1] E[k2] of the kinetic factors, formed in float64 as the library's tables are."""
+    k = np.where(np.arange(n) < (n + 1) // 2, np.arange(n), np.arange(n) - n).astype(float)
+    ph = np.fmod(alpha * k * k * s, 2 * np.pi)
+    re, im = np.cos(ph), -np.sin(ph)
+    return (np.multiply.outer(re, re) - np.multiply.outer(im, im)).ravel(), \
+        (np.multiply.outer(re, im) + np.multiply.outer(im, re)).ravel()
+
+
+def check(multiply, c, s):
+    r = np.random.default_rng(1)
+    x, y = (r.integers(-2 ** 61, 2 ** 61, len(c)).tolist() for _ in range(2))
+    for i, (uc, us, zx, zy) in enumerate(multiply(c, s, x, y)):
+        ec, es = (min(max(float(v), -1.0), 1.0) for v in (c[i], s[i]))
+        assert abs(Fraction(uc, 2 ** 63) - 1 - Fraction(ec)) <= Fraction(1, 2 ** 60), (c[i], uc)
+        assert abs(Fraction(us, 2 ** 63) - 1 - Fraction(es)) <= Fraction(1, 2 ** 60), (s[i], us)
+        fc, fs = Fraction(uc, 2 ** 63) - 1, Fraction(us, 2 ** 63) - 1
+        assert abs(zx - (x[i] * fc - y[i] * fs)) <= 4 and abs(zy - (y[i] * fc + x[i] * fs)) <= 4
+
+
+@pytest.mark.parametrize("n,alpha,s", [(16, 0.05, np.pi), (256, 0.05206503443154336, 0.0068034478138743991),
+                                       (64, 0.05, 2.4166097335306098), (32, 0.5, 2 * np.pi / 40), (32, 0.5, np.pi / 40),
+                                       (64, 0.5, 2 * np.pi / 10), (64, 0.5, np.pi / 10), (128, 0.5, 2 * np.pi / 20)])
+def test_kinetic_factors_near_a_quarter_turn(multiply, n, alpha, s):
+    """Time steps at which factors are 1, i, -1, -i up to rounding: every entry keeps its value."""
+    c, r = pair_table(n, alpha, s)
+    near = np.maximum(np.abs(c), np.abs(r)) >= 1.0 - 2.0 ** -50
+    assert near.any()
+    sel = np.flatnonzero(near)[:2000]
+    check(multiply, c[sel], r[sel])
+
+
+def test_components_at_and_beyond_one(multiply):
+    ulp = 2.0 ** -53
+    v = np.array([1.0, 1 + 2 * ulp, 1 + 4 * ulp, 1 - ulp, 1 - 2 * ulp, 0.0, 2.0 ** -30, 0.7071067811865476])
+    c = np.concatenate([v, -v, np.zeros(16)])
+    s = np.concatenate([np.zeros(16), v, -v])
+    check(multiply, c, s)

@@ -431,16 +431,21 @@ gp_status step_all(gp_plan* p, void* const* psi, int nsteps) {
   }
   const int ncycles = nsteps - 1;
 
+  // in a caller's stream capture only kernels are launched: making a graph inside it is not allowed
+  cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+  GP_CUDA(p, cudaStreamIsCapturing(s, &capturing));
+  const bool direct = p->prof || capturing != cudaStreamCaptureStatusNone;
+
   std::vector<void*> key(psi, psi + p->f.size());
   const long long whole = (long long)pro.size() + (long long)ncycles * (long long)cyc.size() + (long long)tail.size() +
                           (long long)epi.size();
   // a call repeated with the same fields and step count replays one graph of the whole run
-  if (!p->prof && whole <= 8192 && p->run_graph && p->run_key == key && p->run_steps == nsteps) {
+  if (!direct && whole <= 8192 && p->run_graph && p->run_key == key && p->run_steps == nsteps) {
     GP_CUDA(p, cudaGraphLaunch(p->run_graph, s));
     p->launches += whole;
     return GP_OK;
   }
-  if (!p->prof && whole <= 8192 && p->last_key == key && p->last_steps == nsteps) {
+  if (!direct && whole <= 8192 && p->last_key == key && p->last_steps == nsteps) {
     std::vector<std::pair<const std::vector<Item>*, int>> seq = {{&pro, 1}, {&cyc, ncycles}, {&tail, 1}, {&epi, 1}};
     cudaGraphExec_t g = nullptr;
     gp_status st = capture(p, groups, seq, psi, &g);
@@ -453,12 +458,14 @@ gp_status step_all(gp_plan* p, void* const* psi, int nsteps) {
     p->launches += whole;
     return GP_OK;
   }
-  p->last_key = key;
-  p->last_steps = nsteps;
+  if (capturing == cudaStreamCaptureStatusNone) {
+    p->last_key = key;
+    p->last_steps = nsteps;
+  }
 
   gp_status st = run_items(p, groups, pro, psi, s);
   if (st != GP_OK) return st;
-  if (ncycles >= 4 && !p->prof) {
+  if (ncycles >= 4 && !direct) {
     // capture the cycle once per set of field pointers, then replay it
     if (!p->cycle_graph || p->cycle_key != key) {
       if (p->cycle_graph) {

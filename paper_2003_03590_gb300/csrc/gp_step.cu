@@ -166,9 +166,22 @@ bool same_shape(const gp_field_params& a, const gp_field_params& b, const FieldP
          a.nonlin_minus_one == b.nonlin_minus_one && fa.alpha == fb.alpha && fa.beta == fb.beta;
 }
 
-std::vector<Group> make_groups(gp_plan* p) {
+// whether two float64 fields of the plan share memory
+bool f64_shared(gp_plan* p, void* const* psi) {
+  for (size_t i = 0; i < p->f.size(); ++i)
+    for (size_t j = 0; j < i && p->f[i].fp64; ++j) {
+      if (!p->f[j].fp64) continue;
+      const uintptr_t a = (uintptr_t)psi[i], b = (uintptr_t)psi[j];
+      if (a < b + (size_t)p->f[j].npts * sizeof(double2) && b < a + (size_t)p->f[i].npts * sizeof(double2)) return true;
+    }
+  return false;
+}
+
+// f64: float64 fields too
+std::vector<Group> make_groups(gp_plan* p, bool f64) {
   std::vector<Group> g;
   for (int i = 0; i < (int)p->f.size(); ++i) {
+    if (p->f[i].fp64 && !f64) continue;
     bool placed = false;
     for (auto& G : g) {
       const int j = G.fields[0];
@@ -396,7 +409,18 @@ static gp_status fused_batch_steps(gp_plan* p, void* const* psi, int nsteps) {
 gp_status step_all(gp_plan* p, void* const* psi, int nsteps) {
   if (nsteps == 0) return GP_OK;
   if (fused_batch_ok(p)) return fused_batch_steps(p, psi, nsteps);
-  std::vector<Group> groups = make_groups(p);
+  // float64 fields that share memory are advanced one after the other, in the plan's order: the fields
+  // of one launch, and the groups that take turns in the cycle, must not touch each other
+  const bool in_turn = f64_shared(p, psi);
+  if (in_turn) {
+    for (int i = 0; i < (int)p->f.size(); ++i) {
+      if (!p->f[i].fp64) continue;
+      gp_status st = step_field(p, i, psi[i], nsteps);
+      if (st != GP_OK) return st;
+    }
+  }
+  std::vector<Group> groups = make_groups(p, !in_turn);
+  if (groups.empty()) return GP_OK;
   cudaStream_t s = p->stream;
   for (int g = 0; g < (int)groups.size(); ++g) {
     const Group& G = groups[g];

@@ -38,7 +38,7 @@ struct ufix2 {   // a table factor c + i s as ((c + 1) / 2, (s + 1) / 2) in unit
 // a component v of a table factor as ufix2 holds it.  The product of two rounded unit factors can lie an
 // ulp outside [-1, 1]: it counts as 1 or -1 (unclamped, the sum below would wrap to the other sign).
 inline unsigned long long fix_factor(double v) {
-  if (v >= 1.0) return ~1ull;
+  if (!(v < 1.0)) return ~1ull;   // NaN too (see FixArgs::bad)
   if (v <= -1.0) return 0;
   return ((unsigned long long)(long long)std::nearbyint(std::ldexp(v, 62)) << 1) + (1ull << 63);   // (v + 1) 2^63
 }
@@ -245,7 +245,7 @@ inline NlFix nl_fix(double coef, double shift) {
   NlFix f{0, 0, 0, coef < 0.0 ? 1 : 0};
   int e = 0;
   const double mant = std::frexp(std::fabs(coef), &e);          // |coef| = mant 2^e
-  if (mant == 0.0) return f;
+  if (mant == 0.0 || !std::isfinite(coef)) return f;            // (not finite: FixArgs::bad)
   const unsigned long long c = (unsigned long long)std::ldexp(mant, 53) << 11;   // mant 2^64
   // 1 / (2 pi) = 0x28BE60DB9391054A.7F09D5F47D4D3770 2^-64
   typedef unsigned __int128 u128;

@@ -65,6 +65,7 @@ struct Tables {
 struct KTable {
   double s = 0.0;
   void* dev = nullptr;
+  bool finite = true;   // every phase alpha k^2 s is finite
 };
 
 struct FieldPlan {

@@ -227,6 +227,7 @@ const void* ktable(gp_plan* p, int field, double s, bool fp64) {
   ktable_values(F.n, F.alpha, s, re, im);
   KTable kt;
   kt.s = s;
+  for (double v : re) kt.finite = kt.finite && std::isfinite(v);
   cudaError_t e;
   {
     const int n = F.n;
@@ -268,6 +269,8 @@ FixArgs fix_args(FieldPlan& F, const void* ek) {
   a.tw_inv = (const ufix2*)F.t64.tw_inv;
   a.dir = (const ufix2*)F.t64.dir;
   a.ek = (const ufix2*)ek;
+  for (const KTable& k : F.k64)
+    if (k.dev == ek && !k.finite) a.bad = 1;
   return a;
 }
 template <typename T> static auto transform_args(FieldPlan& F) {

@@ -215,6 +215,7 @@ gp_status launch_item(gp_plan* p, const Group& G, const Item& it, void* const* p
     a.op = it.op;
     a.axis = it.axis;
     a.nl = nl_fix(F.beta * it.s_nl, F.prm.nonlin_minus_one ? 1.0 : 0.0);
+    if (!std::isfinite(F.beta * it.s_nl)) a.bad = 1;
     GP_CUDA(p, sweep(G.n, a, s));
     p->launches += 1;
     return GP_OK;

@@ -35,21 +35,31 @@ int main() {
 
 
 @pytest.fixture(scope="module")
-def multiply(tmp_path_factory):
+def host_program(tmp_path_factory):
+    """A function that compiles a C++ source that includes gp_fix.cuh and returns the program's path."""
     cxx = shutil.which("g++") or shutil.which("c++")
     cuda = os.path.join(os.path.dirname(os.path.dirname(shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc")), "include")
     if cxx is None or not os.path.exists(os.path.join(cuda, "cuda_runtime.h")):
         pytest.skip("no host compiler or CUDA headers")
-    d = tmp_path_factory.mktemp("fix")
-    (d / "fix.cpp").write_text(SOURCE)
-    subprocess.run([cxx, "-std=c++17", "-O1", "-I", os.path.join(ROOT, "paper_2003_03590_gb300", "csrc"), "-I", cuda,
-                    str(d / "fix.cpp"), "-o", str(d / "fix")], check=True)
+
+    def build(source):
+        d = tmp_path_factory.mktemp("fix")
+        (d / "fix.cpp").write_text(source)
+        subprocess.run([cxx, "-std=c++17", "-O1", "-I", os.path.join(ROOT, "paper_2003_03590_gb300", "csrc"), "-I", cuda,
+                        str(d / "fix.cpp"), "-o", str(d / "fix")], check=True)
+        return str(d / "fix")
+    return build
+
+
+@pytest.fixture(scope="module")
+def multiply(host_program):
+    prog = host_program(SOURCE)
 
     def run(c, s, x, y):
         bits = [struct.unpack("<Q", struct.pack("<d", v))[0] for v in np.concatenate([c, s])]
         m = len(c)
         text = "".join(f"{bits[i]} {bits[m + i]} {x[i]} {y[i]}\n" for i in range(m))
-        out = subprocess.run([str(d / "fix")], input=text, capture_output=True, text=True, check=True).stdout.split()
+        out = subprocess.run([prog], input=text, capture_output=True, text=True, check=True).stdout.split()
         return [tuple(int(v) for v in out[4 * i:4 * i + 4]) for i in range(m)]
     return run
 
@@ -92,3 +102,19 @@ def test_components_at_and_beyond_one(multiply):
     c = np.concatenate([v, -v, np.zeros(16)])
     s = np.concatenate([np.zeros(16), v, -v])
     check(multiply, c, s)
+
+
+def test_flow_coefficients_that_are_not_finite(host_program):
+    """nl_fix ends for every double (the sweeps then write NaN)."""
+    run = host_program(r"""
+#include <cstdio>
+#include <limits>
+#include "gp_fix.cuh"
+int main() {
+  const double inf = std::numeric_limits<double>::infinity(), nan = std::numeric_limits<double>::quiet_NaN();
+  for (double v : {inf, -inf, nan, 0.0, 5e-324, 1.7e308, -1.7e308})
+    std::printf("%d ", gp::nl_fix(v, 1.0).m >> 63 == 1 ? 1 : 0);
+}
+""")
+    out = subprocess.run([run], capture_output=True, text=True, check=True, timeout=20).stdout
+    assert out.split() == ["0", "0", "0", "0", "1", "1", "1"]

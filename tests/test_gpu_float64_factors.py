@@ -36,3 +36,20 @@ def test_white_field_against_numpy(n, alpha, dt, split):
     ref = np.fft.ifftn(f)
     err = np.linalg.norm(x.cpu().numpy() - ref) / np.linalg.norm(ref)
     assert err <= TOL * (1 if split == GP_SPLIT_NKN else math.sqrt(2)), err
+
+
+@pytest.mark.parametrize("alpha,beta,dt", [(1e300, 0.0, 1e10), (0.05, 1e300, 1e10), (0.05, -1e300, 1e10)])
+@pytest.mark.parametrize("n,split", [(12, GP_SPLIT_NKN), (64, GP_SPLIT_KNK)])
+def test_phases_beyond_the_float64_range_give_nan(alpha, beta, dt, n, split):
+    """Parameters whose phase overflows: NaN, as in float64 arithmetic, in the steps and in the adjoint."""
+    plan = Plan(field_params(n, dt, alpha=alpha, beta=beta, precision=GP_FP64, split=split))
+    start = torch.ones(n, n, n, dtype=torch.complex128, device="cuda")
+    for steps in (1, 6):
+        x = start.clone()
+        plan.step([x], steps)
+        plan.sync()
+        assert bool(torch.view_as_real(x).isnan().all())
+    lam = start.clone()
+    plan.adjoint_step(0, start, lam, 1)
+    plan.sync()
+    assert bool(torch.view_as_real(lam).isnan().any())

@@ -232,13 +232,18 @@ def job_throughput(points_per_rank, steps, world, ms_max):
     return points_per_rank * steps * world / (ms_max / 1e3)
 
 
-def tuned_choices(plan, n):
-    names = {0: "tma", 1: "tma_1cta", 2: "plain", 3: "tma_2stage", 4: "tma_2groups"}
+def fused_plane(roof):
+    """Whether the profiled steps ran y, x, y as the fused plane kernel (roof: roofline_of's record)."""
+    return any(k.startswith("k_tma_plane<") for k in roof["kernels"])
+
+
+def tuned_choices(plan, n, roof):
+    names = {0: "default", 1: "tma_1cta", 2: "plain", 3: "tma_2stage", 4: "tma_other_split", 5: "tma"}
     kinds = {"z:n_fwd": (2, 4), "z:inv_n_fwd": (2, 3), "z:inv_n": (2, 5), "y:fwd": (1, 1), "y:inv": (1, 2),
              "x:fwd_k_inv": (0, 6)}
     out = {k: names.get(plan.sweep_variant(n, a, o), "?") for k, (a, o) in kinds.items()}
     pv = plan.sweep_variant(n, 1, 7)
-    out["y_x_y"] = "three sweeps" if pv == 2 else "fused plane kernel (" + names.get(pv, "?") + ")"
+    out["y_x_y"] = ("fused plane kernel" if fused_plane(roof) else "three sweeps") + " (" + names.get(pv, "?") + ")"
     return out
 
 
@@ -738,7 +743,7 @@ def main():
     roof = roofline_of(gq, plan, psi, n, min(K, 200), peak)
     roof["floor_frac"] = round(floor_frac, 4)
     roof["hbm"]["peak_source"] = peak_src
-    roof["sweeps_per_step"] = 4 if plan.sweep_variant(n, 1, 7) == 2 else 2   # HBM passes of the field
+    roof["sweeps_per_step"] = 2 if fused_plane(roof) else 4   # HBM passes of the field
 
     # end to end through the public C ABI with host buffers
     host = torch.empty((n, n, n), dtype=torch.complex64).pin_memory()
@@ -765,7 +770,7 @@ def main():
             "config": {"workload": f"GP split step {n}^3, xi=1.5dx, dt={DT_MAIN}, RVR {RINGS} rings, fused FP32",
                        "global_batch": world, "seq_len": n ** 3, "parallelism": f"replicas x{world}",
                        "l2": f"field {8 * n ** 3 / 1e6:.0f} MB > 129 MB L2; no flush between steps",
-                       "tuned": tuned_choices(plan, n)},
+                       "tuned": tuned_choices(plan, n, roof)},
             "roofline": roof, "e2e": e2e, "gpu_launches": launches, "clocks": clk, "long_run": long_run}
 
     if not args.no_extras and rank == 0:
@@ -816,8 +821,8 @@ def main():
             r = roofline_of(gq, ps, f, s, min(ks, 20), peak)
             sizes[str(s)] = {"value": s ** 3 * ks / (mss / 1e3), "ms_per_step": mss / ks, "steps": ks,
                              "floor_frac": round(32.0 * s ** 3 / (mss / ks / 1e3) / (peak * 1e9), 4),
-                             "sweeps_per_step": 4 if ps.sweep_variant(s, 1, 7) == 2 else 2,
-                             "tuned": tuned_choices(ps, s), "kinds_mean_us": r["kinds_mean_us"],
+                             "sweeps_per_step": 2 if fused_plane(r) else 4,
+                             "tuned": tuned_choices(ps, s, r), "kinds_mean_us": r["kinds_mean_us"],
                              "dominant": {"kernel": r["kernel"], "time_share": r["time_share"],
                                           "alu_frac": r["frac"], "hbm_frac": r["hbm"]["frac"]}}
             if s >= 1024:

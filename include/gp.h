@@ -229,18 +229,19 @@ long long gp_launch_count(const gp_plan* plan);
  * performs forward y, x (forward, K, inverse) and inverse y of every z-plane in one launch
  * (axis 1).  For every grid length of the plan's float32 fields and every kind of its time step
  * the tuner times the candidates on a scratch field (allocated and freed here) and keeps the
- * fastest: 0 the TMA-pipelined persistent kernel at full occupancy, 1 the same with one CTA per
- * SM, 2 the non-persistent kernel, 3 (y, z and op 7) the TMA kernel with two shared-memory
- * stages, 4 (lengths >= 512, not op 7) the TMA kernel with another split into stages and compute groups; for op 7, 0 = the fused kernel, 1 = the fused kernel with one CTA per SM (fewer planes
- * in flight between its phases), 3 = the fused kernel with two stages, 2 = the three
- * separate sweeps with their own variants.  cache_path (NULL: none) names a JSON file of earlier
+ * fastest.  Variants: 0 the kernel measured fastest for the length when the library was written,
+ * 1 the TMA-pipelined persistent kernel with one CTA per SM, 2 the non-persistent kernel, 3 (y, z
+ * and op 7) the TMA kernel with two shared-memory stages, 4 (lengths >= 512) the TMA kernel with
+ * another split into stages and compute groups, 5 the TMA kernel at full occupancy (the tuner's 0
+ * where it is the default); for op 7, 5 = the fused kernel, 1 = the fused kernel with one CTA per
+ * SM (fewer planes in flight between its phases), 3 and 4 = the fused kernel with two stages and
+ * with several compute groups, 2 = the three separate sweeps with their own variants.  cache_path (NULL: none) names a JSON file of earlier
  * choices keyed by GPU name, length, axis and op; cached choices are reused without timing and
  * new ones are added.  Synchronises the stream and drops captured graphs.
- * gp_plan_sweep_variant returns the variant chosen for a kind by the tuner or by hand (0 if none
- * was: the library then uses, per length, the kernel measured fastest; 2 for lengths without TMA
- * kernels).  gp_plan_set_sweep_variant sets it by hand, 0 included
- * (GP_ERR_INVALID_ARG for an unknown kind or variant); it synchronises the stream and drops
- * captured graphs. */
+ * gp_plan_sweep_variant returns the variant of a kind: the tuner's choice, one set by hand, or 0
+ * (2 for lengths without TMA kernels).  gp_plan_set_sweep_variant sets it by hand, so that setting
+ * what another plan returns gives the other plan's kernels (GP_ERR_INVALID_ARG for an unknown kind
+ * or variant); it synchronises the stream and drops captured graphs. */
 gp_status gp_plan_autotune(gp_plan* plan, const char* cache_path);
 int gp_plan_sweep_variant(gp_plan* plan, int n, int axis, int op);
 gp_status gp_plan_set_sweep_variant(gp_plan* plan, int n, int axis, int op, int variant);

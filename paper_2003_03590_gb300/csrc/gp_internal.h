@@ -137,12 +137,14 @@ FixArgs fix_args(FieldPlan& F, const void* ek);
 cudaError_t launch_nonlinear(double2* psi, long long npts, double coef, double shift, cudaStream_t s);
 cudaError_t launch_vjp_nonlinear(const double2* psi_in, double2* lam, long long npts, double coef, double shift, cudaStream_t s);
 
-// sweep variants (gp_step.cu): 0 TMA persistent, 1 TMA one CTA per SM, 2 plain, 3 TMA with two
-// stages, 4 TMA with another split into stages and compute groups (lengths >= 512); for OP_PLANE 0 means the fused
-// plane kernel, 3 the same with two stages and 2 the three separate sweeps it replaces
-enum { VARIANT_TMA = 0, VARIANT_TMA_ONE = 1, VARIANT_PLAIN = 2, VARIANT_TMA_2STAGE = 3, VARIANT_TMA_GROUPS = 4 };
-int sweep_variant(gp_plan* p, int n, int axis, int op);    // as reported: the plan's choice, or 0
-int kernel_variant(gp_plan* p, int n, int axis, int op);   // as launched: the plan's choice, or the length's
+// sweep variants (gp_step.cu): 0 the kernel measured fastest for the length (what a plan without choices
+// launches), 1 TMA one CTA per SM, 2 plain, 3 TMA with two stages, 4 TMA with another split into stages and
+// compute groups (lengths >= 512), 5 TMA at full occupancy; for OP_PLANE 5 means the fused plane kernel, 1, 3
+// and 4 the same with these variations and 2 the three separate sweeps it replaces
+enum { VARIANT_DEFAULT = 0, VARIANT_TMA_ONE = 1, VARIANT_PLAIN = 2, VARIANT_TMA_2STAGE = 3, VARIANT_TMA_GROUPS = 4, VARIANT_TMA = 5 };
+int sweep_variant(gp_plan* p, int n, int axis, int op);    // as reported and set: VARIANT_DEFAULT included
+int default_variant(int n, int axis, int op);              // what VARIANT_DEFAULT launches
+int kernel_variant(gp_plan* p, int n, int axis, int op);   // as launched
 bool plane_on(gp_plan* p, int n);
 gp_status ensure_plane_sync(gp_plan* p, size_t ints);
 // one float32 sweep of the given kind with the given variant (used by the autotuner)

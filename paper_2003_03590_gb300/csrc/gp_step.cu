@@ -31,10 +31,10 @@ int sweep_variant(gp_plan* p, int n, int axis, int op) {
   const long long k = tune_key(n, axis, op);
   for (const auto& e : p->tune)
     if (e.first == k) return e.second;
-  return VARIANT_TMA;
+  return VARIANT_DEFAULT;
 }
 
-// The kernel of a sweep kind when none was chosen for the plan, by the length.  Measured on GB300, us per
+// The kernel of a sweep kind unless one was chosen for the plan, by the length.  Measured on GB300, us per
 // launch of one field (the batched steps order the same way):
 //   y, x, y as the fused plane kernel / as three sweeps: 32^3 27 / 15, 64^3 29 / 15, 96^3 37 / 23, 128^3
 //     39 / 30, 192^3 103 / 82, 256^3 144 / 153, 512^3 1600 / 1160, 1024^3 11500 / 9240: fused where its
@@ -45,25 +45,22 @@ int sweep_variant(gp_plan* p, int n, int axis, int op) {
 //     of 96^3 251 / 242, of 8 fields of 128^3 220 / 203 (a CTA has few tiles to pipeline); at 192 two
 //     stages: z inverse-N-forward 45.6 / 37.8 / 37.3 (three stages / one tile per CTA / two stages);
 //   z at 1024, TMA / one tile per CTA: forward 3470 / 4900, inverse-N-forward 5440 / 7790.
-static int default_variant(int n, int axis, int op) {
+int default_variant(int n, int axis, int op) {
   if (op == OP_PLANE) return n == 256 ? VARIANT_TMA : VARIANT_PLAIN;
   if (axis == 0 || n <= 128) return VARIANT_PLAIN;
   if (n == 192) return VARIANT_TMA_2STAGE;
   return VARIANT_TMA;
 }
 int kernel_variant(gp_plan* p, int n, int axis, int op) {
-  if (!p->use_tma || !tma_supported(n)) return VARIANT_PLAIN;
-  const long long k = tune_key(n, axis, op);
-  for (const auto& e : p->tune)
-    if (e.first == k) return e.second;
+  const int v = sweep_variant(p, n, axis, op);
+  if (v != VARIANT_DEFAULT) return v;
   if (op == OP_PLANE && p->plane_skip > 0) return VARIANT_TMA;   // gp_plan_test_timeout tests the fused kernel
   return default_variant(n, axis, op);
 }
 
 // forward y, x (forward, K, inverse) and inverse y of a step as one fused plane-kernel launch
 bool plane_on(gp_plan* p, int n) {
-  const int v = kernel_variant(p, n, 1, OP_PLANE);
-  return v == VARIANT_TMA || v == VARIANT_TMA_ONE || v == VARIANT_TMA_2STAGE || v == VARIANT_TMA_GROUPS;
+  return kernel_variant(p, n, 1, OP_PLANE) != VARIANT_PLAIN;
 }
 
 gp_status ensure_plane_sync(gp_plan* p, size_t ints) {
@@ -97,8 +94,7 @@ gp_status ensure_plane_sync(gp_plan* p, size_t ints) {
 cudaError_t launch_sweep_variant(gp_plan* p, int n, const SweepArgs<float>& a, void* const* psi, int variant,
                                  cudaStream_t s) {
   if (a.op == OP_PLANE) {
-    if (variant == VARIANT_TMA || variant == VARIANT_TMA_ONE || variant == VARIANT_TMA_2STAGE ||
-        variant == VARIANT_TMA_GROUPS) {
+    if (variant != VARIANT_PLAIN) {
       const int skip = p->plane_skip;
       p->plane_skip = 0;
       return tma_plane(n, a, psi, p->plane_sync, p->flag + 1, s, variant == VARIANT_TMA_2STAGE ? 2 : 3, skip,

@@ -2,8 +2,9 @@
 //
 // For every grid length of the plan's float32 fields and every sweep kind its time step uses
 // (axis and fused operation), the tuner times the candidate kernels on a scratch field:
-//   0  TMA-pipelined persistent kernel, as many CTAs per SM as fit
-//   1  the same with one CTA per SM (a larger share of L2 and shared-memory bandwidth each)
+//   0  the default, where it is the TMA-pipelined persistent kernel with as many CTAs per SM as fit
+//      (default_variant in gp_step.cu; elsewhere the default is one of the kernels below)
+//   1  that TMA kernel with one CTA per SM (a larger share of L2 and shared-memory bandwidth each)
 //   2  the non-persistent kernel (one tile per CTA, loads and stores by the threads)
 //   3  (y and z) the TMA kernel with two shared-memory stages instead of three: one tile of
 //      look-ahead, one more CTA per SM
@@ -25,15 +26,17 @@ static std::string cache_key(const char* gpu, int n, int axis, int op) {
   return std::string(gpu) + "|" + std::to_string(n) + "|" + std::to_string(axis) + "|" + std::to_string(op);
 }
 
-// candidates per kind: 0-2 everywhere, 3 (two stages) for y, z and the plane kernel; the plane
-// kernel has no one-CTA variant
+// variants of a kind: 0-2 and 5 everywhere, 3 (two stages) for y, z and the plane kernel, 4 from 512 on
 static bool variant_ok(int axis, int op, int v, int n) {
-  if (op == OP_PLANE)
-    return v == VARIANT_TMA || v == VARIANT_TMA_ONE || v == VARIANT_PLAIN || v == VARIANT_TMA_2STAGE ||
-           (v == VARIANT_TMA_GROUPS && n >= 512);
   if (v == VARIANT_TMA_2STAGE) return axis != 0;
   if (v == VARIANT_TMA_GROUPS) return n >= 512;
-  return v >= 0 && v <= 2;
+  return v >= VARIANT_DEFAULT && v <= VARIANT_TMA;
+}
+// the variants the tuner times: each kernel once, so the default only where it is none of the others (the
+// TMA kernel at full occupancy is the default where it is fastest, see default_variant, and not timed elsewhere)
+static bool candidate(int axis, int op, int v, int n) {
+  if (v == VARIANT_DEFAULT) return default_variant(n, axis, op) == VARIANT_TMA;
+  return v != VARIANT_TMA && variant_ok(axis, op, v, n);
 }
 
 // minimal reader/writer for {"key": int, ...}
@@ -89,7 +92,7 @@ extern "C" gp_status gp_plan_autotune(gp_plan* p, const char* cache_path) {
       const long long key = (long long)F.n * 64 + axis * 8 + op;
       int best = -1;
       if (!cache_lookup(text, cache_key(prop.name, F.n, axis, op), &best) || !variant_ok(axis, op, best, F.n)) {
-        best = 0;
+        best = VARIANT_DEFAULT;
         if (!scratch) {
           GP_CUDA(p, cudaMalloc(&scratch, (size_t)F.npts * 8));
           GP_CUDA(p, cudaMemset(scratch, 0, (size_t)F.npts * 8));
@@ -114,9 +117,11 @@ extern "C" gp_status gp_plan_autotune(gp_plan* p, const char* cache_path) {
           if (st != GP_OK) return st;
         }
         float best_ms = 1e30f;
-        for (int var = 0; var < 5; ++var) {
-          if (!variant_ok(axis, op, var, F.n)) continue;
-          auto run = [&]() -> cudaError_t { return launch_sweep_variant(p, F.n, a, &scratch, var, p->stream); };
+        for (int var = VARIANT_DEFAULT; var < VARIANT_TMA; ++var) {
+          if (!candidate(axis, op, var, F.n)) continue;
+          auto run = [&]() -> cudaError_t {
+            return launch_sweep_variant(p, F.n, a, &scratch, var == VARIANT_DEFAULT ? VARIANT_TMA : var, p->stream);
+          };
           for (int w = 0; w < 2; ++w) GP_CUDA(p, run());
           GP_CUDA(p, cudaEventRecord(e0, p->stream));
           for (int r = 0; r < 5; ++r) GP_CUDA(p, run());

@@ -1,12 +1,13 @@
-"""Choices of the float32 sweep kernels, copied from plan to plan.
+"""Choices of the float32 sweep kernels: copied from plan to plan, and every kernel against the plain one.
 
 The kernels a plan launches are read from its profile, not from the numbers it reports.
 """
 import pytest
 import torch
 
-from paper_2003_03590_gb300 import Plan, field_params
-from paper_2003_03590_gb300.gpqt import OP_PLANE, profile, profile_read
+from paper_2003_03590_gb300 import GP_SPLIT_KNK, GP_SPLIT_NKN, Plan, field_params
+from paper_2003_03590_gb300.gpqt import (OP_PLANE, VARIANT_DEFAULT, VARIANT_PLAIN, VARIANT_TMA_2STAGE, VARIANT_TMA_FULL,
+                                         VARIANT_TMA_GROUPS, VARIANT_TMA_ONE, profile, profile_read)
 
 pytestmark = pytest.mark.gpu
 KINDS = [(2, 1), (2, 2), (2, 3), (2, 4), (2, 5), (1, 1), (1, 2), (0, 6), (1, OP_PLANE)]
@@ -38,3 +39,35 @@ def test_copied_choices_give_the_same_kernels(n, tuned):
     for axis, op in KINDS:
         b.set_sweep_variant(n, axis, op, a.sweep_variant(n, axis, op))
     assert _launched(a, _start(n)) == _launched(b, _start(n))
+
+
+@pytest.mark.parametrize("split", [GP_SPLIT_NKN, GP_SPLIT_KNK])
+@pytest.mark.parametrize("n", [32, 48, 64, 96, 128, 192, 256, 512, 1024])
+def test_every_kernel_equals_the_plain_one(n, split):
+    start = _start(n)
+    variants = [VARIANT_PLAIN, VARIANT_DEFAULT, VARIANT_TMA_FULL, VARIANT_TMA_ONE, VARIANT_TMA_2STAGE]
+    if n >= 512:
+        variants.append(VARIANT_TMA_GROUPS)
+    ref = None
+    for fused in (False, True):
+        for v in variants:
+            if fused and v == VARIANT_PLAIN:
+                continue
+            plan = Plan(field_params(n, 0.001, xi_over_dx=1.5, split=split))
+            for axis, op in KINDS:
+                if op == OP_PLANE:
+                    plan.set_sweep_variant(n, axis, op, v if fused else VARIANT_PLAIN)
+                elif not (v == VARIANT_TMA_2STAGE and axis == 0):
+                    plan.set_sweep_variant(n, axis, op, v)
+            x = start.clone()
+            names = {k.split("<")[0] for k in _launched(plan, x)}
+            if v == VARIANT_PLAIN:
+                assert all(k.startswith("k_sweep_") for k in names), names
+                ref = x
+            else:
+                assert torch.equal(x, ref), (v, fused)
+                if v != VARIANT_DEFAULT:
+                    assert ("k_tma_plane" in names) == fused
+                    assert not any(k.startswith("k_sweep_strided") for k in names), (v, names)
+            del plan, x
+    torch.cuda.empty_cache()

@@ -236,7 +236,7 @@ long long gp_launch_count(const gp_plan* plan);
  * where it is the default); for op 7, 5 = the fused kernel, 1 = the fused kernel with one CTA per
  * SM (fewer planes in flight between its phases), 3 and 4 = the fused kernel with two stages and
  * with several compute groups, 2 = the three separate sweeps with their own variants.  cache_path (NULL: none) names a JSON file of earlier
- * choices keyed by GPU name, length, axis and op; cached choices are reused without timing and
+ * choices keyed by GPU name, version of the kernels, length, axis and op; cached choices are reused without timing and
  * new ones are added.  Synchronises the stream and drops captured graphs.
  * gp_plan_sweep_variant returns the variant of a kind: the tuner's choice, one set by hand, or 0
  * (2 for lengths without TMA kernels).  gp_plan_set_sweep_variant sets it by hand, so that setting

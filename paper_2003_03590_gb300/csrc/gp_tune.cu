@@ -11,7 +11,7 @@
 //   4  (lengths from 512 on) the TMA kernel with another split into stages and compute groups
 // (at 1024 every TMA variant of z is the one kernel of gp_ztile.cuh)
 // and keeps the fastest; the fused plane kernel (op 7) is timed against the three sweeps it
-// replaces.  Choices are cached in a small JSON file keyed by the GPU's name.
+// replaces.  Choices are cached in a small JSON file keyed by the GPU's name and the kernels' version.
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -22,8 +22,12 @@
 
 namespace gp {
 
+// Version of the kernels behind the variant numbers, raised whenever one of them changes: a choice timed on
+// other kernels is not reused (files without a version named 2 for z at 1024, now 1.4 times slower than 0).
+constexpr int KERNELS_VERSION = 2;
+
 static std::string cache_key(const char* gpu, int n, int axis, int op) {
-  return std::string(gpu) + "|" + std::to_string(n) + "|" + std::to_string(axis) + "|" + std::to_string(op);
+  return std::string(gpu) + "|v" + std::to_string(KERNELS_VERSION) + "|" + std::to_string(n) + "|" + std::to_string(axis) + "|" + std::to_string(op);
 }
 
 // variants of a kind: 0-2 and 5 everywhere, 3 (two stages) for y, z and the plane kernel, 4 from 512 on
@@ -152,7 +156,7 @@ extern "C" gp_status gp_plan_autotune(gp_plan* p, const char* cache_path) {
     (void)timed;
   }
   if (cache_path && !out_entries.empty()) {
-    // keep the entries of other GPUs and lengths already in the file
+    // keep the entries of other GPUs, versions and lengths already in the file
     std::string merged = "{\n" + out_entries;
     size_t pos = 0;
     while ((pos = text.find('"', pos)) != std::string::npos) {

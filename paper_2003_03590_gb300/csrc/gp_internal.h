@@ -26,6 +26,8 @@ struct TmaPlaneArgs;
 GP_TMA_SIZES(GP_DECL_TMA)
 #undef GP_DECL_TMA
 bool tma_supported(int n);
+const char* tma_kernel_name(int n, int axis);     // of a TMA variant's sweep, "name<"
+const char* plain_kernel_name(int n, int axis);   // of the plain variant's
 // launch one TMA sweep for the fields psi[0..count) of length n (float32 fused path)
 cudaError_t tma_sweep(int n, const SweepArgs<float>& a, void* const* psi, int* status, cudaStream_t s,
                       int ctas_req = 0,    // CTAs per SM; 0: as many as fit

@@ -47,6 +47,17 @@ cudaError_t sweep(int n, const SweepArgs<float>& a, cudaStream_t s) {
     default: return cudaErrorInvalidValue;
   }
 }
+const char* plain_kernel_name(int n, int axis) {
+  switch (n) {
+#define GP_CASE(L)                                                                       \
+  case L:                                                                                \
+    if (sweep_capped<float, L>()) return axis == 0 ? "k_sweep_contig_rc<float," : "k_sweep_strided_rc<float,"; \
+    return axis == 0 ? "k_sweep_contig<float," : "k_sweep_strided<float,";
+    GP_SIZES(GP_CASE)
+#undef GP_CASE
+    default: return "";
+  }
+}
 cudaError_t sweep(int n, const FixArgs& a, cudaStream_t s) {
   switch (n) {
 #define GP_CASE(L) case L: return sweep_f64_##L(a, s);

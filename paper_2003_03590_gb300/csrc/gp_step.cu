@@ -237,11 +237,7 @@ gp_status launch_item(gp_plan* p, const Group& G, const Item& it, void* const* p
     static const char* opn[] = {"", "fwd", "inv", "inv_n_fwd", "n_fwd", "inv_n", "fwd_k_inv", "fwd_k_inv"};
     const bool tma = kernel_variant(p, G.n, it.axis, it.op) != VARIANT_PLAIN;
     std::string name = it.op == OP_PLANE ? std::string("k_tma_plane<") + std::to_string(G.n) + ">:y_fwd_x_fwd_k_inv_y_inv:xy"
-                       : std::string(tma ? (G.n >= 256 && !(G.n == 512 && it.axis == 1) ? "k_warp_sweep<"
-                                            : it.axis == 0 ? "k_tma_contig<" : "k_tma_strided<")
-                                         : G.n >= 512 ? (it.axis == 0 ? "k_sweep_contig_rc<float," : "k_sweep_strided_rc<float,")
-                                                      : (it.axis == 0 ? "k_sweep_contig<float," : "k_sweep_strided<float,")) +
-                             std::to_string(G.n) + ">:" + opn[it.op] + ":" + "xyz"[it.axis];
+                       : std::string(tma ? tma_kernel_name(G.n, it.axis) : plain_kernel_name(G.n, it.axis)) + std::to_string(G.n) + ">:" + opn[it.op] + ":" + "xyz"[it.axis];
     int kind = -1;
     for (int q = 0; q < (int)p->kinds.size(); ++q)
       if (p->kinds[q] == name) kind = q;

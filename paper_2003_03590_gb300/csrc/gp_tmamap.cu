@@ -19,6 +19,20 @@ bool tma_supported(int n) {
   }
 }
 
+template <int L> static const char* kernel_name(int axis) {
+  if (ztile_ok<L>() && axis == 2) return "k_ztile<";
+  if (warp_axis<L>(axis)) return "k_warp_sweep<";
+  return axis == 0 ? "k_tma_contig<" : "k_tma_strided<";
+}
+const char* tma_kernel_name(int n, int axis) {
+  switch (n) {
+#define GP_CASE(L) case L: return kernel_name<L>(axis);
+    GP_TMA_SIZES(GP_CASE)
+#undef GP_CASE
+    default: return "";
+  }
+}
+
 static PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   if (!fn) {

@@ -71,3 +71,22 @@ def test_every_kernel_equals_the_plain_one(n, split):
                     assert not any(k.startswith("k_sweep_strided") for k in names), (v, names)
             del plan, x
     torch.cuda.empty_cache()
+
+
+@pytest.mark.parametrize("n", [32, 96, 192, 256, 512, 1024])
+def test_profile_names_the_kernels(n):
+    tail = "_rc" if n >= 512 or n in (96, 192) else ""
+    want = {VARIANT_PLAIN: {"x": f"k_sweep_contig{tail}<float,{n}>", "y": f"k_sweep_strided{tail}<float,{n}>",
+                            "z": f"k_sweep_strided{tail}<float,{n}>"},
+            VARIANT_TMA_FULL: {"x": f"k_warp_sweep<{n}>" if n >= 256 else f"k_tma_contig<{n}>",
+                               "y": f"k_warp_sweep<{n}>" if n in (256, 1024) else f"k_tma_strided<{n}>",
+                               "z": f"k_ztile<{n}>" if n == 1024 else f"k_warp_sweep<{n}>" if n >= 256 else f"k_tma_strided<{n}>"}}
+    for v, names in want.items():
+        plan = Plan(field_params(n, 0.001, xi_over_dx=1.5)).set_sweep_variant(n, 1, OP_PLANE, VARIANT_PLAIN)
+        for axis, op in KINDS[:-1]:
+            plan.set_sweep_variant(n, axis, op, v)
+        got = {}
+        for k in _launched(plan, _start(n)):
+            kernel, _, axis = k.split(":")
+            got.setdefault(axis, set()).add(kernel)
+        assert got == {a: {k} for a, k in names.items()}

@@ -11,6 +11,7 @@
 //   RVR pairs     pair p: positions 4p..4p+3 -> shift X, Y, Z (2 pi u) and axis order floor(6u)
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 #include <vector>
 
 #include "gp_internal.h"
@@ -202,7 +203,7 @@ struct Ring {
 
 // A float64-like number in two floats (hi + lo, about 46 bits) for float32 fields: this GPU has 64
 // float32 lanes for each float64 one.  The sums and products are the usual error-free ones
-// (Knuth's two-sum, the fma product remainder).
+// (Knuth's two-sum, the fma product remainder); each is off by at most 2^-46 of its operands' size.
 struct Twofold {
   float h, l;
 };
@@ -240,18 +241,20 @@ __device__ __forceinline__ Twofold make_num(double v, Twofold*) {
   return Twofold{h, (float)(v - (double)h)};
 }
 
-__device__ __forceinline__ Twofold scaled(Twofold a, float b) { return mulf(a, b); }
-__device__ __forceinline__ double scaled(double a, float b) { return a * (double)b; }
-__device__ __forceinline__ double add(double a, double b) { return a + b; }
-__device__ __forceinline__ double neg(double a) { return -a; }
-__device__ __forceinline__ double mul(double a, double b) { return a * b; }
-__device__ __forceinline__ double sqr(double a) { return a * a; }
+__device__ __forceinline__ Twofold madd(Twofold a, Twofold b, Twofold c) { return add(mul(a, b), c); }    // a b + c
+__device__ __forceinline__ Twofold msub(Twofold a, Twofold b, Twofold c) { return add(c, neg(mul(a, b))); }   // c - a b
+__device__ __forceinline__ bool positive(Twofold a) { return a.h > 0.0f; }
+
+// the same in float64, every rounding written out, so that every kernel that uses them rounds alike
+__device__ __forceinline__ double add(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double sqr(double a) { return __dmul_rn(a, a); }
+__device__ __forceinline__ double madd(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ double msub(double a, double b, double c) { return __fma_rn(-a, b, c); }
 __device__ __forceinline__ double inv_sqrt(double x) { return rsqrt(x); }
 __device__ __forceinline__ float lead(double a) { return (float)a; }
 __device__ __forceinline__ double value(double a) { return a; }
 __device__ __forceinline__ double make_num(double v, double*) { return v; }
-
-__device__ __forceinline__ bool positive(Twofold a) { return a.h > 0.0f; }
 __device__ __forceinline__ bool positive(double a) { return a > 0.0; }
 
 template <typename Num> struct RingNum {
@@ -274,48 +277,104 @@ __global__ void k_ring_tables(const Ring* __restrict__ rings, int count, int n, 
   }
 }
 
-// One point per thread, the rings in turn.  Bound by arithmetic: about 260 float32 operations per point
-// and ring (float32 fields), 45 float64 ones (float64 fields).  256^3, 40 rings, float32 field on
-// GB300: 98.6 ms with every operation in float64 (and divisions, floors and square roots per point),
-// 7.7 ms now, the same 2.1e-8 (the rounding of the output) from float64 arithmetic.
-template <typename T, typename Num>
-__global__ void __launch_bounds__(256) k_rings(const RingNum<Num>* __restrict__ rings, const Num* __restrict__ tab, int count, int n, double xi, cpx<T>* psi) {
+// The field of the rings at one point.  err (Twofold): a bound of the error of re and im.
+// Bound of a ring's factor F = tanh(s / (sqrt 2 xi)) / s (rho' - R, z'), in units of 2^-46: z' takes six roundings of
+// numbers up to 5.4 (the largest displacement), 19; the projected displacement another 45; rho' and its difference from R
+// 30 + 1.25 R; so (rho' - R, z') is off by at most 75 + 1.25 R, and F by tanh(.) / s, its steepest slope, times that
+// and by 40 for its own roundings and the product with the rings before.  A half more throughout.
+template <typename Num>
+__device__ __forceinline__ void ring_point(const RingNum<Num>* __restrict__ rings, const Num* __restrict__ tab, int count, int n, double xi,
+                                           long long i, Num& re, Num& im, float& err) {
+  constexpr bool TWO = std::is_same<Num, Twofold>::value;
   Num* const none = nullptr;
-  const long long npts = (long long)n * n * n;
   const float inv = (float)(1.0 / (sqrt(2.0) * xi));
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < npts; i += (long long)gridDim.x * blockDim.x) {
-    const int ix = (int)(i % n), iy = (int)((i / n) % n), iz = (int)(i / ((long long)n * n));
-    Num re = make_num(1.0, none), im = make_num(0.0, none);
-    for (int j = 0; j < count; ++j) {
-      const Num* dj = tab + (long long)j * 3 * n;
-      const Num d0 = dj[ix], d1 = dj[n + iy], d2 = dj[2 * n + iz];
-      const RingNum<Num> g = rings[j];
-      const Num zp = add(add(mul(d0, g.n0), mul(d1, g.n1)), mul(d2, g.n2));
-      const Num p0 = add(d0, neg(mul(zp, g.n0))), p1 = add(d1, neg(mul(zp, g.n1))), p2 = add(d2, neg(mul(zp, g.n2)));
-      const Num r2 = add(add(sqr(p0), sqr(p1)), sqr(p2));
-      const Num rp = positive(r2) ? mul(r2, inv_sqrt(r2)) : r2;
-      const Num rr = add(rp, g.minus_R);
-      const Num s2 = add(sqr(rr), sqr(zp));
-      // tanh(s / (sqrt 2 xi)) exp(i atan2(z', rho' - R)) = tanh(.) (rho' - R + i z') / s: the phase
-      // factor is the unit vector of the core offset; at s = 0 the amplitude is 0
-      Num f = make_num(0.0, none);
-      if (positive(s2)) {
-        f = inv_sqrt(s2);
-        const float sa = sqrtf(lead(s2)) * inv;
-        // beyond 22 core widths tanh is 1 to far below an ulp; float32 fields: from 10 on 1 - tanh =
-        // 2 exp(-2 s) below 5e-9, by float32
-        if (sizeof(Num) == sizeof(Twofold) && sizeof(T) == 4 && sa >= 10.0f) {
-          if (sa < 22.0f) f = add(f, scaled(f, -2.0f * expf(-2.0f * sa)));
-        } else if (sa < 22.0f) {
-          f = mul(f, make_num(tanh(sqrt(value(s2)) * (1.0 / (sqrt(2.0) * xi))), none));
-        }
+  const int ix = (int)(i % n), iy = (int)((i / n) % n), iz = (int)(i / ((long long)n * n));
+  re = make_num(1.0, none), im = make_num(0.0, none);
+  err = 0.0f;
+  for (int j = 0; j < count; ++j) {
+    const Num* dj = tab + (long long)j * 3 * n;
+    const Num d0 = dj[ix], d1 = dj[n + iy], d2 = dj[2 * n + iz];
+    const RingNum<Num> g = rings[j];
+    const Num zp = madd(d2, g.n2, madd(d1, g.n1, mul(d0, g.n0)));
+    const Num p0 = msub(zp, g.n0, d0), p1 = msub(zp, g.n1, d1), p2 = msub(zp, g.n2, d2);
+    const Num r2 = madd(p2, p2, madd(p1, p1, sqr(p0)));
+    const Num rp = positive(r2) ? mul(r2, inv_sqrt(r2)) : r2;
+    const Num rr = add(rp, g.minus_R);
+    const Num s2 = madd(zp, zp, sqr(rr));
+    // tanh(s / (sqrt 2 xi)) exp(i atan2(z', rho' - R)) = tanh(.) (rho' - R + i z') / s: the phase
+    // factor is the unit vector of the core offset; at s = 0 the amplitude is 0
+    Num f = make_num(0.0, none);
+    float slope = inv;
+    if (positive(s2)) {
+      f = inv_sqrt(s2);
+      const float sa = sqrtf(lead(s2)) * inv;
+      // beyond 22 core widths tanh is 1 to far below an ulp; twofold: from 10 on 1 - tanh = 2 exp(-2 s)
+      // below 5e-9, by float32
+      if (TWO && sa >= 10.0f) {
+        if constexpr (TWO)
+          if (sa < 22.0f) f = add(f, mulf(f, -2.0f * expf(-2.0f * sa)));
+      } else if (sa < 22.0f) {
+        f = mul(f, make_num(tanh(sqrt(value(s2)) * (1.0 / (sqrt(2.0) * xi))), none));
       }
-      const Num fr = mul(f, rr), fi = mul(f, zp);
-      const Num nr = add(mul(re, fr), neg(mul(im, fi))), ni = add(mul(re, fi), mul(im, fr));
-      re = nr;
-      im = ni;
+      slope = lead(f);
     }
-    psi[i] = cpx<T>{(T)value(re), (T)value(im)};
+    if constexpr (TWO) err = fmaf(slope, fmaf(1.6f, fabsf(g.minus_R.h), 112.0f), err + 60.0f);
+    const Num fr = mul(f, rr), fi = mul(f, zp);
+    const Num nr = msub(im, fi, mul(re, fr)), ni = madd(im, fr, mul(re, fi));
+    re = nr;
+    im = ni;
+  }
+  err = err * 0x1p-46f;
+}
+
+// One point per thread, the rings in turn.  Bound by arithmetic: about 260 float32 operations per point
+// and ring in twofold numbers, 45 float64 ones.  GB300, 256^3, 40 rings, float32 field: 98.6 ms with every operation in
+// float64 (and divisions, floors and square roots per point), 7.7 ms for this kernel in twofold numbers and 1.1 ms
+// for the points in doubt.  Their share grows with the rings: 1000 rings 479 ms, of which 191 here (all in float64: 1029).
+// doubt (Twofold): one bit per point whose rounded value the error bound leaves open; k_rings_doubt forms those in
+// float64, so that a float32 field is the float64 one rounded, bit for bit.
+template <typename T, typename Num>
+__global__ void __launch_bounds__(256) k_rings(const RingNum<Num>* __restrict__ rings, const Num* __restrict__ tab, int count, int n, double xi, cpx<T>* psi, unsigned* doubt) {
+  const long long npts = (long long)n * n * n;   // a multiple of 64: whole warps
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < npts; i += (long long)gridDim.x * blockDim.x) {
+    Num re, im;
+    float err;
+    ring_point(rings, tab, count, n, xi, i, re, im, err);
+    if constexpr (std::is_same<Num, Twofold>::value) {
+      // the low part is below 2^-24 of the high one: forming low +- err is off by less than a unit of err
+      const float r = __fadd_rn(re.h, re.l - err), m = __fadd_rn(im.h, im.l - err);
+      psi[i] = float2{r, m};
+      const bool open = !(r == __fadd_rn(re.h, re.l + err) && m == __fadd_rn(im.h, im.l + err));
+      const unsigned bits = __ballot_sync(0xffffffffu, open);
+      if ((threadIdx.x & 31) == 0) doubt[i >> 5] = bits;
+    } else {
+      psi[i] = cpx<T>{(T)re, (T)im};
+    }
+  }
+}
+// The points in doubt of `points` (a multiple of 32) consecutive points per block: their numbers are gathered
+// first, so that warps are full.
+constexpr int DOUBT_POINTS = 8192;   // at most
+template <typename T>
+__global__ void __launch_bounds__(256) k_rings_doubt(const RingNum<double>* __restrict__ rings, const double* __restrict__ tab, int count, int n, double xi,
+                                                     cpx<T>* psi, const unsigned* __restrict__ doubt, int points) {
+  __shared__ unsigned short list[DOUBT_POINTS];
+  __shared__ int used;
+  const long long base = (long long)blockIdx.x * points, npts = (long long)n * n * n;
+  if (threadIdx.x == 0) used = 0;
+  __syncthreads();
+  for (int w = threadIdx.x; w < points / 32 && base + 32ll * w < npts; w += blockDim.x) {
+    unsigned bits = doubt[(base >> 5) + w];
+    int at = bits ? atomicAdd(&used, __popc(bits)) : 0;
+    for (; bits; bits &= bits - 1) list[at++] = (unsigned short)(32 * w + __ffs(bits) - 1);
+  }
+  __syncthreads();
+  for (int q = threadIdx.x; q < used; q += blockDim.x) {
+    const long long i = base + list[q];
+    double re, im;
+    float err;
+    ring_point(rings, tab, count, n, xi, i, re, im, err);
+    psi[i] = cpx<T>{(T)re, (T)im};
   }
 }
 
@@ -443,20 +502,40 @@ static void box_muller(uint64_t va, uint64_t vb, double* g0, double* g1) {
   *g1 = r * std::sin(t);
 }
 
-template <typename T, typename Num>
-static gp_status rings_field(gp_plan* p, int field, cpx<T>* psi, const std::vector<Ring>& rings, int count, double xi) {
+template <typename T>
+static gp_status rings_field(gp_plan* p, int field, cpx<T>* psi, const std::vector<Ring>& rings, int count, double xi, bool twofold) {
   FieldPlan& F = p->f[field];
-  const size_t rb = (rings.size() * sizeof(Ring) + 15) / 16 * 16;
-  const size_t nb = rings.size() * sizeof(RingNum<Num>);
-  gp_status st = ensure_ws(p, field, rb + nb + rings.size() * 3 * F.n * sizeof(Num));
+  const size_t m = rings.size(), entries = m * 3 * F.n;
+  // the rings; float64: their numbers and the displacements; twofold: the same, and the points in doubt
+  const size_t rb = (m * sizeof(Ring) + 15) / 16 * 16, nb = m * sizeof(RingNum<double>), mb = m * sizeof(RingNum<Twofold>);
+  gp_status st = ensure_ws(p, field, rb + nb + entries * sizeof(double) +
+                                         (twofold ? mb + entries * sizeof(Twofold) + (size_t)F.npts / 8 : 0));
   if (st != GP_OK) return st;
   cudaStream_t s = p->stream;
   GP_CUDA(p, cudaMemcpyAsync(F.ws, rings.data(), rings.size() * sizeof(Ring), cudaMemcpyHostToDevice, s));
-  RingNum<Num>* rn = (RingNum<Num>*)((unsigned char*)F.ws + rb);
-  Num* tab = (Num*)((unsigned char*)rn + nb);
-  if (count > 0) k_ring_tables<Num><<<(3 * F.n * count + 255) / 256, 256, 0, s>>>((const Ring*)F.ws, count, F.n, rn, tab);
+  const Ring* dev = (const Ring*)F.ws;
+  RingNum<double>* rn = (RingNum<double>*)((unsigned char*)F.ws + rb);
+  double* tab = (double*)((unsigned char*)rn + nb);
+  const unsigned tg = (unsigned)((entries + 255) / 256);
+  if (count > 0) k_ring_tables<double><<<tg, 256, 0, s>>>(dev, count, F.n, rn, tab);
   GP_CUDA(p, cudaGetLastError());
-  k_rings<T, Num><<<igrid(F.npts), 256, 0, s>>>(rn, tab, count, F.n, xi, psi);
+  if (!twofold) {
+    k_rings<T, double><<<igrid(F.npts), 256, 0, s>>>(rn, tab, count, F.n, xi, psi, nullptr);
+  } else if constexpr (sizeof(T) == 4) {
+    RingNum<Twofold>* rn2 = (RingNum<Twofold>*)(tab + entries);
+    Twofold* tab2 = (Twofold*)((unsigned char*)rn2 + mb);
+    unsigned* doubt = (unsigned*)(tab2 + entries);
+    if (count > 0) k_ring_tables<Twofold><<<tg, 256, 0, s>>>(dev, count, F.n, rn2, tab2);
+    GP_CUDA(p, cudaGetLastError());
+    k_rings<T, Twofold><<<igrid(F.npts), 256, 0, s>>>(rn2, tab2, count, F.n, xi, psi, doubt);
+    GP_CUDA(p, cudaGetLastError());
+    // four blocks per SM or more; small fields have few points a block (their time is one point's chain of float64
+    // operations)
+    long long points = (F.npts / (152 * 4) + 255) / 256 * 256;
+    if (points > DOUBT_POINTS) points = DOUBT_POINTS;
+    if (points < 256) points = 256;
+    k_rings_doubt<T><<<(unsigned)((F.npts + points - 1) / points), 256, 0, s>>>(rn, tab, count, F.n, xi, psi, doubt, (int)points);
+  }
   GP_CUDA(p, cudaGetLastError());
   GP_CUDA(p, cudaStreamSynchronize(s));
   return GP_OK;
@@ -487,7 +566,7 @@ static gp_status rvr_rings(gp_plan* p, int field, cpx<T>* psi, uint64_t seed, in
   // the box, a core far wider or narrower than any grid)
   bool twofold = sizeof(T) == 4 && xi > 1e-6 && xi < 1e4;
   for (const Ring& g : rings) twofold = twofold && std::fabs(g.R) < 1e4;
-  return twofold ? rings_field<T, Twofold>(p, field, psi, rings, count, xi) : rings_field<T, double>(p, field, psi, rings, count, xi);
+  return rings_field<T>(p, field, psi, rings, count, xi, twofold);
 }
 template <typename T>
 static gp_status rvr_pairs(gp_plan* p, int field, cpx<T>* psi, uint64_t seed, int npairs, double R, double d) {

@@ -29,21 +29,11 @@ template <> struct CT<float> { using v = float2; };
 template <> struct CT<double> { using v = double2; };
 template <typename T> using cpx = typename CT<T>::v;
 
-template <typename V> __device__ __forceinline__ V cadd(V a, V b) { return V{a.x + b.x, a.y + b.y}; }
-template <typename V> __device__ __forceinline__ V csub(V a, V b) { return V{a.x - b.x, a.y - b.y}; }
-// float32: one packed FP32x2 instruction per complex operation.  Each lane rounds exactly as the
+// one packed FP32x2 instruction per complex operation.  Each lane rounds exactly as the
 // scalar operation would (b * -1 is exact, so fma(b, -1, a) is a - b rounded once).
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return __ffma2_rn(b, float2{-1.0f, -1.0f}, a); }
 __device__ __forceinline__ float2 swap2(float2 a) { return float2{a.y, a.x}; }
-template <typename V> __device__ __forceinline__ V cmul(V a, V b) {
-  return V{a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
-}
-template <typename V> __device__ __forceinline__ V cmulconj(V a, V b) {  // a * conj(b)
-  return V{a.x * b.x + a.y * b.y, a.y * b.x - a.x * b.y};
-}
-template <typename V, typename S> __device__ __forceinline__ V cscale(V a, S s) { return V{a.x * s, a.y * s}; }
-__device__ __forceinline__ float2 cscale(float2 a, float s) { return __fmul2_rn(a, float2{s, s}); }
 template <typename V> __device__ __forceinline__ V cneg(V a) { return V{-a.x, -a.y}; }
 // a * (-i) for the forward direction, a * (+i) for the inverse one
 template <bool INV, typename V> __device__ __forceinline__ V mul_mi(V a) {
@@ -55,16 +45,14 @@ template <bool INV, typename V> __device__ __forceinline__ V mul_mi(V a) {
 // fixed relative error of the rounded constant.  A fixed error would bias |w|^2
 // the same way in every step and make the mass (conserved exactly by the
 // scheme) drift linearly in time; the compensated product leaves only unbiased
-// round-off.  float64 uses the constant directly.
+// round-off.
 struct KConst {
-  double v;
   float hi, lo;
 };
 __host__ __device__ constexpr KConst kconst(double v) {
-  return KConst{v, (float)v, (float)(v - (double)(float)v)};
+  return KConst{(float)v, (float)(v - (double)(float)v)};
 }
 __device__ __forceinline__ float kmul(float x, KConst k) { return fmaf(x, k.hi, x * k.lo); }
-__device__ __forceinline__ double kmul(double x, KConst k) { return x * k.v; }
 // both lanes of a float2 times the constants sa * k (lane 0) and sb * k (lane 1), sa, sb = +-1:
 // per lane fma(x, +-hi, x * +-lo), the negation of kmul(x, k) when the sign is -1
 __device__ __forceinline__ float2 kmul2(float2 x, KConst k, float sa, float sb) {
@@ -72,49 +60,35 @@ __device__ __forceinline__ float2 kmul2(float2 x, KConst k, float sa, float sb) 
 }
 
 // a * (c - i s) forward, a * (c + i s) inverse, for constants c = cos(theta), s = sin(theta)
-// (float: every product-sum is an explicit fma, so that the rounding does not depend on how the
+// (every product-sum is an explicit fma, so that the rounding does not depend on how the
 // compiler would contract a*b + c*d in a given kernel -- all kernel variants agree bitwise)
-// NEG: the negated product (float: the constants negated, which rounds to exactly the negation).
-template <bool INV, typename V, bool NEG = false> __device__ __forceinline__ V rotk(V a, KConst c, KConst s) {
-  if constexpr (sizeof(a.x) == 4) {
-    // lanes (re, im): lo = a c.lo + (+-a.y, -+a.x) s.lo;  result = a c.hi + ((+-a.y, -+a.x) s.hi + lo)
-    const float2 b = swap2(a);
-    const float sg = INV ? -1.0f : 1.0f, ng = NEG ? -1.0f : 1.0f;
-    const float2 lo = __ffma2_rn(a, float2{ng * c.lo, ng * c.lo}, __fmul2_rn(b, float2{ng * sg * s.lo, -ng * sg * s.lo}));
-    return __ffma2_rn(a, float2{ng * c.hi, ng * c.hi}, __ffma2_rn(b, float2{ng * sg * s.hi, -ng * sg * s.hi}, lo));
-  } else {
-    const V r = INV ? V{a.x * c.v - a.y * s.v, a.y * c.v + a.x * s.v} : V{a.x * c.v + a.y * s.v, a.y * c.v - a.x * s.v};
-    return NEG ? cneg(r) : r;
-  }
+// NEG: the negated product (the constants negated, which rounds to exactly the negation).
+template <bool INV, bool NEG = false> __device__ __forceinline__ float2 rotk(float2 a, KConst c, KConst s) {
+  // lanes (re, im): lo = a c.lo + (+-a.y, -+a.x) s.lo;  result = a c.hi + ((+-a.y, -+a.x) s.hi + lo)
+  const float2 b = swap2(a);
+  const float sg = INV ? -1.0f : 1.0f, ng = NEG ? -1.0f : 1.0f;
+  const float2 lo = __ffma2_rn(a, float2{ng * c.lo, ng * c.lo}, __fmul2_rn(b, float2{ng * sg * s.lo, -ng * sg * s.lo}));
+  return __ffma2_rn(a, float2{ng * c.hi, ng * c.hi}, __ffma2_rn(b, float2{ng * sg * s.hi, -ng * sg * s.hi}, lo));
 }
 // multiplication by exp(-+ i pi/4) and exp(-+ 3 i pi/4): one constant, 1/sqrt(2)
 constexpr KConst K_R2 = kconst(0.70710678118654752440);
 constexpr KConst K_C16 = kconst(0.92387953251128675613);   // cos(pi/8)
 constexpr KConst K_S16 = kconst(0.38268343236508977173);   // sin(pi/8)
 constexpr KConst K_H3 = kconst(0.86602540378443864676);    // sqrt(3)/2
-template <bool INV, typename V> __device__ __forceinline__ V rot45(V a) {   // * exp(-+ i pi/4)
-  if constexpr (sizeof(a.x) == 4) {
-    // forward (a.x + a.y, -(a.x - a.y)) K;  inverse (a.x - a.y, a.x + a.y) K
-    if constexpr (INV) return kmul2(__ffma2_rn(swap2(a), float2{-1.0f, 1.0f}, a), K_R2, 1.0f, 1.0f);
-    else return kmul2(__ffma2_rn(a, float2{1.0f, -1.0f}, swap2(a)), K_R2, 1.0f, -1.0f);
-  } else {
-    return INV ? V{kmul(a.x - a.y, K_R2), kmul(a.x + a.y, K_R2)} : V{kmul(a.x + a.y, K_R2), kmul(a.y - a.x, K_R2)};
-  }
+template <bool INV> __device__ __forceinline__ float2 rot45(float2 a) {   // * exp(-+ i pi/4)
+  // forward (a.x + a.y, -(a.x - a.y)) K;  inverse (a.x - a.y, a.x + a.y) K
+  if constexpr (INV) return kmul2(__ffma2_rn(swap2(a), float2{-1.0f, 1.0f}, a), K_R2, 1.0f, 1.0f);
+  else return kmul2(__ffma2_rn(a, float2{1.0f, -1.0f}, swap2(a)), K_R2, 1.0f, -1.0f);
 }
-template <bool INV, typename V> __device__ __forceinline__ V rot135(V a) {  // * exp(-+ 3 i pi/4)
-  if constexpr (sizeof(a.x) == 4) {
-    // forward (a.y - a.x, -(a.x + a.y)) K;  inverse (-(a.x + a.y), a.x - a.y) K
-    if constexpr (INV) return kmul2(__ffma2_rn(a, float2{1.0f, -1.0f}, swap2(a)), K_R2, -1.0f, 1.0f);
-    else return kmul2(__ffma2_rn(a, float2{-1.0f, 1.0f}, swap2(a)), K_R2, 1.0f, -1.0f);
-  } else {
-    return INV ? V{kmul(-a.x - a.y, K_R2), kmul(a.x - a.y, K_R2)} : V{kmul(a.y - a.x, K_R2), kmul(-a.x - a.y, K_R2)};
-  }
+template <bool INV> __device__ __forceinline__ float2 rot135(float2 a) {  // * exp(-+ 3 i pi/4)
+  // forward (a.y - a.x, -(a.x + a.y)) K;  inverse (-(a.x + a.y), a.x - a.y) K
+  if constexpr (INV) return kmul2(__ffma2_rn(a, float2{1.0f, -1.0f}, swap2(a)), K_R2, -1.0f, 1.0f);
+  else return kmul2(__ffma2_rn(a, float2{-1.0f, 1.0f}, swap2(a)), K_R2, 1.0f, -1.0f);
 }
 
-// Stockham twiddle storage: float32 keeps hi (x, y) and lo (z, w) parts, float64 the value.
+// Stockham twiddle storage: hi (x, y) and lo (z, w) parts (float64 fields: gp_fix.cuh).
 template <typename T> struct TwT;
 template <> struct TwT<float> { using v = float4; };
-template <> struct TwT<double> { using v = double2; };
 template <typename T> using tw_t = typename TwT<T>::v;
 
 __device__ __forceinline__ float2 twmul(float2 a, float4 w) {   // a * (w.hi + w.lo), one rounding
@@ -122,7 +96,6 @@ __device__ __forceinline__ float2 twmul(float2 a, float4 w) {   // a * (w.hi + w
   const float im_lo = fmaf(a.x, w.w, a.y * w.z);
   return float2{fmaf(a.x, w.x, fmaf(-a.y, w.y, re_lo)), fmaf(a.x, w.y, fmaf(a.y, w.x, im_lo))};
 }
-__device__ __forceinline__ double2 twmul(double2 a, double2 w) { return cmul(a, w); }
 // a * w as twmul, but with the larger of the two products of each component added last.  The
 // kinetic factor turns a slowly rotating mode by the same tiny angle at every step; summing its
 // small terms against the larger product alone first (as twmul's imaginary part does) would round
@@ -154,8 +127,6 @@ __device__ __forceinline__ float2 unit_rotate(float2 v, float c, float s) {
   const float im = fmaf(v.x, s, fmaf(v.y, c, fmaf(v.x, ds, v.y * dc)));
   return float2{re, im};
 }
-__device__ __forceinline__ double2 unit_rotate(double2 v, double c, double s) { return cmul(v, double2{c, s}); }
-
 
 // ---------------------------------------------------------------- butterflies
 // In-register DFTs of size 2, 3, 4, 8, 16, 32, natural order in and out.
@@ -166,17 +137,11 @@ template <bool INV, typename V> __device__ __forceinline__ void dft2(V& a, V& b)
 }
 
 // p = e + m, q = e - m with m = -+i o (forward -i, inverse +i)
-template <bool INV, typename V> __device__ __forceinline__ void add_sub_mi(V e, V o, V& p, V& q) {
-  if constexpr (sizeof(e.x) == 4) {
-    // -i o = (o.y, -o.x), i o = (-o.y, o.x): both lanes from the swapped o with signs
-    const float2 os = swap2(o);
-    p = __ffma2_rn(os, INV ? float2{-1.0f, 1.0f} : float2{1.0f, -1.0f}, e);
-    q = __ffma2_rn(os, INV ? float2{1.0f, -1.0f} : float2{-1.0f, 1.0f}, e);
-  } else {
-    const V m = mul_mi<INV>(o);
-    p = cadd(e, m);
-    q = csub(e, m);
-  }
+template <bool INV> __device__ __forceinline__ void add_sub_mi(float2 e, float2 o, float2& p, float2& q) {
+  // -i o = (o.y, -o.x), i o = (-o.y, o.x): both lanes from the swapped o with signs
+  const float2 os = swap2(o);
+  p = __ffma2_rn(os, INV ? float2{-1.0f, 1.0f} : float2{1.0f, -1.0f}, e);
+  q = __ffma2_rn(os, INV ? float2{1.0f, -1.0f} : float2{-1.0f, 1.0f}, e);
 }
 
 template <bool INV, typename V> __device__ __forceinline__ void dft4(V& a0, V& a1, V& a2, V& a3) {
@@ -187,17 +152,10 @@ template <bool INV, typename V> __device__ __forceinline__ void dft4(V& a0, V& a
 }
 
 template <bool INV, typename V> __device__ __forceinline__ void dft3(V& a0, V& a1, V& a2) {
-  using S = decltype(a0.x);
   V t1 = cadd(a1, a2);
   V d = csub(a1, a2);
-  V t2, t3;
-  if constexpr (sizeof(S) == 4) {
-    t2 = __ffma2_rn(t1, float2{-0.5f, -0.5f}, a0);   // a0 - t1 / 2 (the product is exact)
-    t3 = kmul2(d, K_H3, 1.0f, 1.0f);                  // (a1 - a2) sqrt(3)/2
-  } else {
-    t2 = V{a0.x - S(0.5) * t1.x, a0.y - S(0.5) * t1.y};
-    t3 = V{kmul(d.x, K_H3), kmul(d.y, K_H3)};
-  }
+  V t2 = __ffma2_rn(t1, float2{-0.5f, -0.5f}, a0);   // a0 - t1 / 2 (the product is exact)
+  V t3 = kmul2(d, K_H3, 1.0f, 1.0f);                  // (a1 - a2) sqrt(3)/2
   V it3 = V{-t3.y, t3.x};  // i t3
   a0 = cadd(a0, t1);
   if (!INV) { a1 = csub(t2, it3); a2 = cadd(t2, it3); }
@@ -230,7 +188,7 @@ template <bool INV, typename V> __device__ __forceinline__ void dft16(V* v) {
   v[11] = rot135<INV>(v[11]);              // n2=3,k1=2: w^6
   v[13] = rotk<INV>(v[13], K_S16, K_C16);  // n2=1,k1=3: w^3
   v[14] = rot135<INV>(v[14]);              // n2=2,k1=3: w^6
-  v[15] = rotk<INV, V, true>(v[15], K_C16, K_S16);  // n2=3,k1=3: w^9 = -w^1
+  v[15] = rotk<INV, true>(v[15], K_C16, K_S16);  // n2=3,k1=3: w^9 = -w^1
 #pragma unroll
   for (int k1 = 0; k1 < 4; ++k1) dft4<INV>(v[4 * k1], v[4 * k1 + 1], v[4 * k1 + 2], v[4 * k1 + 3]);
   // v[4 k1 + k2] = X[k1 + 4 k2]: transpose to natural order

@@ -96,7 +96,6 @@ __device__ __forceinline__ void red_release_gpu_add(int* p, int v) {
 }
 __device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait1() { asm volatile("cp.async.bulk.wait_group 1;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait2() { asm volatile("cp.async.bulk.wait_group 2;" ::: "memory"); }
 
 // Item order.  Blocks of Q items (one phase of one plane) are ordered by "group" g: group g
 // holds phase 0 of plane g, phase 1 of plane g - D and phase 2 of plane g - 2D (those that
@@ -415,7 +414,7 @@ __global__ void __launch_bounds__(TmaPlane<L, NS, NG>::NT, TmaPlane<L, NS, NG>::
   }
 }
 
-// compute groups and stages of the grouped plane kernel: 512: three groups, five stages;
+// compute groups and stages of the grouped plane kernel: 512: four groups, six stages;
 // 1024: two groups, three stages (a 1024-point stage is 70 KB)
 template <int L> __host__ __device__ constexpr int plane_groups() { return L >= 1024 ? 2 : 4; }
 template <int L> __host__ __device__ constexpr int plane_group_stages() { return L >= 1024 ? 3 : 6; }

@@ -118,3 +118,99 @@ int main() {
 """)
     out = subprocess.run([run], capture_output=True, text=True, check=True, timeout=20).stdout
     assert out.split() == ["0", "0", "0", "0", "1", "1", "1"]
+
+
+CONVERT = r"""
+#include <cstdio>
+#include "gp_fix.cuh"
+// "t bits s": to_fix; "f v s": from_fix
+int main() {
+  char k;
+  unsigned long long u;
+  int s;
+  while (std::scanf(" %c %llu %d", &k, &u, &s) == 3)
+    std::printf("%lld\n", k == 't' ? gp::to_fix(u, s) : (long long)gp::from_fix((long long)u, s));
+}
+"""
+
+
+def test_conversions_round_to_nearest_even(host_program):
+    """float64 to fixed point and back: the nearest number, ties to even, over the float64 range."""
+    prog = host_program(CONVERT)
+    r = np.random.default_rng(2)
+    lines, want = [], []
+    for _ in range(3000):
+        d = float(r.standard_normal() * 2.0 ** r.integers(-1000, 960))
+        e = int(np.frexp(d)[1])
+        s = int(61 - e - r.integers(0, 70))                  # |d| 2^s < 2^62, down to less than a unit
+        lines.append(f"t {struct.unpack('<Q', struct.pack('<d', d))[0]} {s}")
+        want.append(round(Fraction(d) * Fraction(2) ** s))
+        v = int(r.integers(-2 ** 62, 2 ** 62)) >> int(r.integers(0, 62))
+        s = int(r.integers(-900, 900))
+        lines.append(f"f {v % 2 ** 64} {s}")
+        want.append(struct.unpack("<q", struct.pack("<d", float(Fraction(v) * Fraction(2) ** -s)))[0])
+    # ties: 53 bits and a half
+    for k in range(64):
+        v = ((2 ** 52 + k) << 11) + 2 ** 10
+        lines.append(f"f {v - 2 ** 62 if v >= 2 ** 63 else v} 0")
+        want.append(struct.unpack("<q", struct.pack("<d", float(v - 2 ** 62 if v >= 2 ** 63 else v)))[0])
+    out = subprocess.run([prog], input="\n".join(lines), capture_output=True, text=True, check=True).stdout.split()
+    assert [int(x) for x in out] == want
+
+
+FLOW = r"""
+#include <cmath>
+#include <cstdio>
+#include "gp_fix.cuh"
+static unsigned long long factor(long double v) {   // (v + 1) 2^63, even
+  const long double u = (v + 1.0L) * 4611686018427387904.0L;
+  return u >= 9223372036854775807.0L ? ~1ull : (unsigned long long)std::nearbyintl(u) << 1;
+}
+// "coef shift x y s": exp(-i coef (|psi|^2 - shift)) psi for psi = (x + i y) 2^-s, in units of 2^-s
+int main() {
+  gp::ufix2 dir[256];
+  const long double pi = 3.14159265358979323846264338327950288L;
+  for (int k = 0; k < 256; ++k) dir[k] = gp::ufix2{factor(cosl(2 * pi * k / 256)), factor(sinl(2 * pi * k / 256))};
+  double coef, shift;
+  long long x, y;
+  int s;
+  while (std::scanf("%lf %lf %lld %lld %d", &coef, &shift, &x, &y, &s) == 5) {
+    const gp::NlFix f = gp::nl_fix(coef, shift);
+    const gp::cfix z = gp::fnonlinear(gp::cfix{x, y}, 2 * s + f.q - 126, f.m, f.tc, f.neg, dir);
+    std::printf("%lld %lld\n", z.x, z.y);
+  }
+}
+"""
+
+
+def test_nonlinear_flow_against_extended_precision(host_program):
+    """N(s) at one point, |psi|^2 from 1e-12 to 100 and |coef| |psi|^2 up to 20.
+
+    At the kernels' scale the larger component has 62 bits, |psi|^2 then 61 and two truncations: the phase is good to
+    2^-59 |coef| |psi|^2 (float64: 2^-53); the directions, the products and the series add a few 2^-61, 1e-17 in all.
+    Needs a long double of 64 bits or more.
+    """
+    if np.finfo(np.longdouble).nmant < 63:
+        pytest.skip("long double is double here")
+    prog = host_program(FLOW)
+    r = np.random.default_rng(3)
+    ext = np.longdouble
+    cases = []
+    for _ in range(2000):
+        amp = 10.0 ** r.uniform(-6, 1)
+        ph = r.uniform(0, 2 * np.pi)
+        re, im = amp * np.cos(ph), amp * np.sin(ph)
+        s = int(62 - np.frexp(max(abs(re), abs(im)))[1])
+        x, y = int(re * 2.0 ** s), int(im * 2.0 ** s)
+        coef = float(r.uniform(-20, 20) / max(amp * amp, 1.0))
+        cases.append((coef, float(r.integers(0, 2)), x, y, s))
+    text = "".join(f"{c!r} {h!r} {x} {y} {s}\n" for c, h, x, y, s in cases)
+    out = subprocess.run([prog], input=text, capture_output=True, text=True, check=True).stdout.split()
+    for i, (c, h, x, y, s) in enumerate(cases):
+        u = ext(2) ** ext(-s)
+        X, Y = ext(x) * u, ext(y) * u
+        ph = ext(c) * (X * X + Y * Y - ext(h))
+        cs, sn = np.cos(ph), np.sin(ph)
+        err = np.hypot(ext(int(out[2 * i])) * u - (X * cs + Y * sn), ext(int(out[2 * i + 1])) * u - (Y * cs - X * sn))
+        bound = (ext(2) ** -59 * abs(c) * (X * X + Y * Y) + 1e-17) * np.hypot(X, Y)
+        assert err <= bound, (cases[i], float(err / np.hypot(X, Y)))

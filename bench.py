@@ -18,7 +18,7 @@ Metric: N^3 * steps / s (grid points advanced per second), whole job.  Also repo
   e2e          the same metric through gp_step_host with the field in pinned host memory,
                one host->device copy, one step and one device->host copy per bench step
   cpu_baseline the float64 numpy oracle, one full 256^3 step, on the host
-  fp64_plain   the unfused complex128 GPU path, cufft_torch the cuFFT + elementwise baseline
+  fp64_plain   the complex128 GPU path (fixed-point sweeps), cufft_torch the cuFFT + elementwise baseline
   sizes        512^3 and 1024^3 (smoothed-random-phase start, k0 = 8, dt = 0.001)
 N > 1 GPUs (torchrun): every rank advances its own independent field (replicas; the
 ensemble shards without communication), value = all ranks' points * steps / max time.
@@ -81,12 +81,16 @@ def kernel_source_hash():
 
 
 def records_current(lines):
-    """False if the records name another source of gp_warp.cuh (lines: # gp_warp.cuh <sha256, 16 digits>)."""
+    """False if the records name another source of a header (lines: # <header>.cuh <sha256, 16 digits>)."""
     for line in lines:
         m = line.split()
-        if m[:2] == ["#", "gp_warp.cuh"]:
-            with open(os.path.join(ROOT, "paper_2003_03590_gb300", "csrc", "gp_warp.cuh"), "rb") as fh:
-                return hashlib.sha256(fh.read()).hexdigest()[:16] == m[2]
+        if len(m) == 3 and m[0] == "#" and m[1].endswith(".cuh"):
+            path = os.path.join(ROOT, "paper_2003_03590_gb300", "csrc", m[1])
+            if not os.path.exists(path):
+                return False
+            with open(path, "rb") as fh:
+                if hashlib.sha256(fh.read()).hexdigest()[:16] != m[2]:
+                    return False
     return True
 
 

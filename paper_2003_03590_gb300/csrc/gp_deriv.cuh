@@ -11,7 +11,7 @@
 // A CTA walks tiles of pencils of one axis (gp_sweep.cuh's tiles and transforms).  The next tile is
 // copied to shared memory (cp.async) while the current one is worked on, and stays there for the
 // pointwise work; the exchanges between radix passes use a buffer of their own.  Bound by latency and
-// instruction issue at 16 warps per SM (128 registers a thread): GB300, 256^3, the diagnostics' three
+// instruction issue at 16 warps per SM (128 registers a thread; 12 at 96 and 192, see deriv_ahead): GB300, 256^3, the diagnostics' three
 // kernels (3 or 4 transforms and 20 to 28 bytes per point each) 0.15, 0.15 and 0.22 ms.
 #pragma once
 #include <type_traits>
@@ -44,14 +44,16 @@ template <int L, bool CONTIG> __host__ __device__ constexpr int deriv_batch() {
   return CONTIG ? contig_batch<float, L>() : strided_batch<float, L>();
 }
 template <int L, bool CONTIG> __host__ __device__ constexpr int deriv_threads() { return deriv_batch<L, CONTIG>() * (L / Plan<L>::E); }
-// CTAs per SM that the registers must allow: 16 warps per SM
+// CTAs per SM that the registers must allow (16 warps per SM)
 template <int L, bool CONTIG> __host__ __device__ constexpr int deriv_min_ctas() {
   return 512 / deriv_threads<L, CONTIG>() > 16 ? 16 : 512 / deriv_threads<L, CONTIG>();
 }
 template <int L, bool CONTIG> __host__ __device__ constexpr int deriv_exchange() {   // elements
   return (CONTIG ? contig_pitch<L>() : L) * deriv_batch<L, CONTIG>();
 }
-// two tiles of look-ahead fit (with those CTAs) up to 256 points; beyond, one tile at a time, read directly
+// two tiles of look-ahead up to 256 points; beyond, one tile at a time, read directly.  With those CTAs they fit in
+// shared memory, but for the lengths of 24 elements a thread: 96 and 192 hold three quarters of them (192 three CTAs of
+// 74 to 77 KB, 96 three of 77 KB for x and six of 37 KB for y and z), 12 warps per SM
 template <int L> __host__ __device__ constexpr bool deriv_ahead() { return L >= 32 && L <= 256; }
 template <int L, bool CONTIG> __host__ __device__ constexpr size_t deriv_smem() {
   return sizeof(float2) * ((size_t)deriv_exchange<L, CONTIG>() + (deriv_ahead<L>() ? 2 * (size_t)deriv_batch<L, CONTIG>() * L : 0));
@@ -171,7 +173,7 @@ template <int L, class EPI> cudaError_t deriv_launch(const DerivArgs& a, const E
   static const cudaError_t attr = cudaFuncSetAttribute(k_deriv<L, EPI>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (attr != cudaSuccess) return attr;
   const int tiles = L * L / deriv_batch<L, CONTIG>();
-  // whole rounds of the CTAs that fit; at most DERIV_BLOCKS
+  // as many as the registers allow at once, DERIV_BLOCKS at most (at 192 the last quarter runs after the others)
   int blocks = 152 * deriv_min_ctas<L, CONTIG>();
   if (blocks > DERIV_BLOCKS) blocks = DERIV_BLOCKS;
   k_deriv<L, EPI><<<tiles < blocks ? tiles : blocks, deriv_threads<L, CONTIG>(), smem, s>>>(a, tiles, epi);

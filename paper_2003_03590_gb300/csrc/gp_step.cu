@@ -130,7 +130,7 @@ cudaError_t fft1_many(gp_plan* p, FieldPlan& F, cpx<float>* const* xs, int count
   return launch_sweep_variant(p, F.n, a, ptrs, kernel_variant(p, F.n, a.axis, a.op), s);
 }
 // 3D transforms of `count` float32 fields of one plan length, one launch per axis for all of
-// them, through the kernel variants chosen for the forward and inverse y/z sweeps (x: TMA)
+// them, through the kernel variants chosen for the forward and inverse y/z sweeps (x: the default, plain)
 cudaError_t fft3_many(gp_plan* p, FieldPlan& F, cpx<float>* const* xs, int count, bool inverse, cudaStream_t s) {
   const int order_f[3] = {0, 1, 2}, order_i[3] = {2, 1, 0};
   for (int i = 0; i < 3; ++i) {

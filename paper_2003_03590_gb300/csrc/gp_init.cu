@@ -563,8 +563,10 @@ static gp_status rvr_rings(gp_plan* p, int field, cpx<T>* psi, uint64_t seed, in
   }
   const double xi = std::sqrt(F.alpha / F.beta);
   // float32 fields: twofold float32, unless the lengths would leave its range (a ring far larger than
-  // the box, a core far wider or narrower than any grid)
-  bool twofold = sizeof(T) == 4 && xi > 1e-6 && xi < 1e4;
+  // the box, a core far wider or narrower than any grid), or the field has less than a block of points per SM:
+  // then the time is one point's chain of operations and two more launches, and float64 is faster (GB300, 1, 5 and 40
+  // rings, us, twofold / float64: 32^3 40, 66, 278 / 29, 49, 221; 48^3 47, 92, 430 / 39, 96, 596; 64^3 54, 110, 550 / 59, 193, 1345)
+  bool twofold = sizeof(T) == 4 && xi > 1e-6 && xi < 1e4 && F.npts > 152 * 256;
   for (const Ring& g : rings) twofold = twofold && std::fabs(g.R) < 1e4;
   return rings_field<T>(p, field, psi, rings, count, xi, twofold);
 }

@@ -13,7 +13,7 @@ from paper_2003_03590_gb300 import GP_FP32, GP_FP64, Plan, field_params
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n", [8, 12, 24, 64, 96, 128, 192, 256])
+@pytest.mark.parametrize("n", [8, 12, 24, 32, 48, 64, 96, 128, 192, 256])
 @pytest.mark.parametrize("count,r0,r1,xi_dx", [(0, 1.0, 2.0, 1.5), (1, 0.0, 0.0, 1.5), (5, 4.0, 12.0, 2.0), (40, 4.0, 12.0, 1.5),
                                                (400, 4.0, 12.0, 1.5), (7, 1.0, 60.0, 0.05), (5, 2.0, 3.0, 40.0),
                                                (3, -8.0, 8.0, 1.5), (3, 1e7, 2e7, 1.5), (4096, 2.0, 6.0, 0.3)])

@@ -302,6 +302,10 @@ static gp_status adjoint_f32(gp_plan* p, int field, const float2* psi_n, float2*
   FieldPlan& F = p->f[field];
   const long long npts = F.npts;
   cudaStream_t s = p->stream;
+  // every table before the first change of lam
+  const bool nkn = F.prm.split == GP_SPLIT_NKN;
+  for (double t : {nkn ? F.prm.dt : 0.5 * F.prm.dt, F.prm.dt})
+    if (!ktable(p, field, t, false) || !ktable(p, field, -t, false)) return fail(p, GP_ERR_OOM, "kinetic table allocation");
   // the work field and nsteps - 1 states; a copy of psi_n where lam, written from the first sweep back on, overlaps it
   const bool overlap = psi_n < lam + npts && lam < psi_n + npts;
   const size_t need = (size_t)(nsteps + overlap) * (size_t)npts * sizeof(float2);
@@ -328,7 +332,7 @@ static gp_status adjoint_f32(gp_plan* p, int field, const float2* psi_n, float2*
     z.src = src, z.dst = dst, z.out = out, z.state = nullptr, z.c1 = c1, z.c2 = c2;
   };
   auto vjp = [&](const float2* S, float c1, float c2) { z.src = z.dst = lam, z.out = nullptr, z.state = S, z.c1 = c1, z.c2 = c2; };
-  if (F.prm.split == GP_SPLIT_NKN) {
+  if (nkn) {
     // states S_1 .. S_{n-1} into their slots, S_n into work
     flow(psi_n, work, nullptr, 0.0f, ch);
     GP_CUDA(p, (adj_z<Z_STATE, false, true>(F.n, z, s)));

@@ -406,6 +406,9 @@ gp_status step_all(gp_plan* p, void* const* psi, int nsteps) {
   // of one launch, and the groups that take turns in the cycle, must not touch each other
   const bool in_turn = f64_shared(p, psi);
   if (in_turn) {
+    for (int i = 0; i < (int)p->f.size(); ++i)   // tables first: no field changes if one cannot be had
+      if (p->f[i].fp64 && (!ktable(p, i, p->f[i].prm.dt, true) || !ktable(p, i, 0.5 * p->f[i].prm.dt, true)))
+        return fail(p, GP_ERR_OOM, "kinetic table allocation");
     for (int i = 0; i < (int)p->f.size(); ++i) {
       if (!p->f[i].fp64) continue;
       gp_status st = step_field(p, i, psi[i], nsteps);

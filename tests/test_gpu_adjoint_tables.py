@@ -46,3 +46,36 @@ def test_cotangent_kept_when_tables_are_missing(prec, dtype, split):
     plan.step([psi.clone(), psi.clone()], 1)
     plan.sync()
     assert status == 3 and kept                             # GP_ERR_OOM
+
+
+def test_shared_float64_fields_kept_when_tables_are_missing():
+    """The same for float64 fields that share memory: the second field's tables cannot be had, the first has its own."""
+    n = 32
+    plan = Plan([field_params(n, dt, xi_over_dx=1.5, precision=GP_FP64) for dt in (0.004, 0.002)], stream=torch.cuda.Stream())
+    x = torch.full((n, n, n), 0.5 + 0.25j, dtype=torch.complex128, device="cuda")
+    torch.cuda.synchronize()
+    plan.adjoint_step(0, x.clone(), x.clone(), 1)           # the first field's tables
+    plan.sync()
+    keep = x.clone()
+    torch.cuda.synchronize()
+    graph, other = torch.cuda.CUDAGraph(), torch.cuda.Stream()
+    status = None
+    with torch.cuda.stream(other):
+        graph.capture_begin()
+        try:
+            plan.step([x, x], 2)
+        except GPError as e:
+            status = e.status
+        try:
+            graph.capture_end()
+        except Exception:  # noqa: BLE001
+            pass
+    torch.cuda.synchronize()
+    kept = torch.equal(x, keep)
+    try:
+        plan.step([x, x], 1)                                # reports the refused allocation's pending error
+    except GPError:
+        pass
+    plan.step([x, x], 1)
+    plan.sync()
+    assert status == 3 and kept

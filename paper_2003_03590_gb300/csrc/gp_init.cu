@@ -203,7 +203,9 @@ struct Ring {
 
 // A float64-like number in two floats (hi + lo, about 46 bits) for float32 fields: this GPU has 64
 // float32 lanes for each float64 one.  The sums and products are the usual error-free ones
-// (Knuth's two-sum, the fma product remainder); each is off by at most 2^-46 of its operands' size.
+// (Knuth's two-sum, the fma product remainder).  With u = 2^-24 a sum is off by at most 3 u^2 (|a| + |b|) (the low
+// parts' sum and its sum with the remainder, each rounded once), a product by 6 u^2 |a b| (three roundings of numbers
+// below u, 2 u and 3 u, and the low parts' product left out), inv_sqrt by 19 u^2 of its value.
 struct Twofold {
   float h, l;
 };
@@ -278,10 +280,14 @@ __global__ void k_ring_tables(const Ring* __restrict__ rings, int count, int n, 
 }
 
 // The field of the rings at one point.  err (Twofold): a bound of the error of re and im.
-// Bound of a ring's factor F = tanh(s / (sqrt 2 xi)) / s (rho' - R, z'), in units of 2^-46: z' takes six roundings of
-// numbers up to 5.4 (the largest displacement), 19; the projected displacement another 45; rho' and its difference from R
-// 30 + 1.25 R; so (rho' - R, z') is off by at most 75 + 1.25 R, and F by tanh(.) / s, its steepest slope, times that
-// and by 40 for its own roundings and the product with the rings before.  A half more throughout.
+// Bound, in units of u^2 = 2^-48 (Twofold), |d| <= 5.44 the displacement, d and the normal n stored to 1 each:
+//   z' = d . n: 8 per product, 6 per sum, of 5.44 in all                                      76
+//   d - z' n: z' and 14 more of 5.44                                                         152
+//   rho' = r2 r2^-1/2: (12 / 2 + 19 + 6) 5.44                                                169
+//   rho' - R: 3 (5.44 + R) + R                                                          16 + 4 R
+// so (rho' - R, z') is off by at most 345 + 4 R, and the ring's factor F = tanh(.) / s (rho' - R, z') by that times
+// tanh(.) / s, its steepest slope, and by 39 |F| for its own operations; the product with the rings before adds 9.  Below, in
+// units of 2^-46 and a sixth more: (100 + 1.2 R) tanh(.) / s + 20.
 template <typename Num>
 __device__ __forceinline__ void ring_point(const RingNum<Num>* __restrict__ rings, const Num* __restrict__ tab, int count, int n, double xi,
                                            long long i, Num& re, Num& im, float& err) {
@@ -318,7 +324,7 @@ __device__ __forceinline__ void ring_point(const RingNum<Num>* __restrict__ ring
       }
       slope = lead(f);
     }
-    if constexpr (TWO) err = fmaf(slope, fmaf(1.6f, fabsf(g.minus_R.h), 112.0f), err + 60.0f);
+    if constexpr (TWO) err = fmaf(slope, fmaf(1.2f, fabsf(g.minus_R.h), 100.0f), err + 20.0f);
     const Num fr = mul(f, rr), fi = mul(f, zp);
     const Num nr = msub(im, fi, mul(re, fr)), ni = madd(im, fr, mul(re, fi));
     re = nr;
@@ -329,8 +335,8 @@ __device__ __forceinline__ void ring_point(const RingNum<Num>* __restrict__ ring
 
 // One point per thread, the rings in turn.  Bound by arithmetic: about 260 float32 operations per point
 // and ring in twofold numbers, 45 float64 ones.  GB300, 256^3, 40 rings, float32 field: 98.6 ms with every operation in
-// float64 (and divisions, floors and square roots per point), 7.7 ms for this kernel in twofold numbers and 1.1 ms
-// for the points in doubt.  Their share grows with the rings: 1000 rings 479 ms, of which 191 here (all in float64: 1029).
+// float64 (and divisions, floors and square roots per point), 7.7 ms for this kernel in twofold numbers and 0.9 ms
+// for the points in doubt.  Their share grows with the rings: 1000 rings 389 ms, of which 191 here (all in float64: 1030).
 // doubt (Twofold): one bit per point whose rounded value the error bound leaves open; k_rings_doubt forms those in
 // float64, so that a float32 field is the float64 one rounded, bit for bit.
 template <typename T, typename Num>

@@ -25,7 +25,7 @@ struct FixArgs {
   const ufix2* dir;        // the 256 directions of gp_fix.cuh's fnonlinear
   NlFix nl;
   int op, axis;
-  int bad;                 // 1: the flow's phase is not finite: every value becomes NaN, as float64 arithmetic has it
+  int bad;                 // 1: the flow's phase is not finite; no kernel is launched, sweep() writes NaN
   int scale_inv;           // 1: inverse ops multiply by 1/N; 0: normalisation done with K (1/N^3)
 };
 
@@ -212,7 +212,7 @@ __device__ __forceinline__ void fix_op(const FixArgs& a, int t, int p, cfix* sm,
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = cfix{rescale1(v[e].x, r), rescale1(v[e].y, r)};
   };
-  const bool bad = s == FIX_NOT_FINITE || a.bad;   // every value of the pencil becomes NaN
+  const bool bad = s == FIX_NOT_FINITE;   // every value of the pencil becomes NaN
   if (bad) s = 0;
   {
     const int s0 = OP == OP_N_FWD ? 1084 - ref : s;

@@ -59,6 +59,13 @@ const char* plain_kernel_name(int n, int axis) {
   }
 }
 cudaError_t sweep(int n, const FixArgs& a, cudaStream_t s) {
+  if (a.bad) {   // every value becomes NaN, as in float64 arithmetic (all bits set is one)
+    for (int k = 0; k < a.count; ++k) {
+      const cudaError_t e = cudaMemsetAsync(a.psi[k], 0xff, sizeof(double2) * (size_t)n * n * n, s);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+  }
   switch (n) {
 #define GP_CASE(L) case L: return sweep_f64_##L(a, s);
     GP_SIZES(GP_CASE)
